@@ -163,8 +163,10 @@ gals_status gals_set_state(gals_grid *grid, const float *const *fields, int nfie
  * device and advances it, so longer calls replay the same graph.  In 2D the graph splits each step into up to 4 bands of whole tile
  * rows, at least 2 tiles and the velocity's reach plus 4 rows high; a band of step s
  * depends only on itself and its two neighbouring bands at step s - 1, so the next step's
- * bands start while the current one drains (same results bit for bit).  Asynchronous on
- * the grid stream.
+ * bands start while the current one drains (same results bit for bit).  A run of 8 or more
+ * steps on a 2D grid of at most 12288 nodes (rows of at most 512) is one launch of a
+ * thread-block cluster that keeps the state in shared memory (bit for bit too).
+ * Asynchronous on the grid stream.
  * Errors: GALS_ERR_ARG (dt <= 0 or non-finite, nsteps < 0, bad velocity descriptor),
  * GALS_ERR_STATE (no state loaded), GALS_ERR_UNSUPPORTED (velocity kind not available in
  * this dimension), GALS_ERR_CUDA (launch failure). */

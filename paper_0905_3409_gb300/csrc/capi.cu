@@ -191,6 +191,14 @@ bool use_run(const gals_grid *g, int trace, int nsteps, const double reach[2])
            reach[0] <= run2d_max_cells(0) && reach[1] <= run2d_max_cells(1);
 }
 
+// Whether a run of nsteps steps is one cluster launch (launch_step2d_small): a small 2D grid
+// and an analytic trace, in the default time loop.
+bool use_small(const gals_grid *g, int trace, int nsteps)
+{
+    return g->loop == GALS_LOOP_LAUNCHES && g->dim == 2 && nsteps >= kSmallSteps && trace != GALS_TRACE_SURROGATE &&
+           small2d_fits(g->geom);
+}
+
 // Row bands of a captured multi-step 2D call.  Step s of band b reads the rows of step
 // s - 1 that its feet reach (plus the staged tile's halo row and the cubic cell) and
 // overwrites rows that step s - 1 of the neighbouring bands read, so with bands at least
@@ -327,6 +335,30 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
         launches += (g->dim == 3 && a.write_cross) ? 2 : 1;  // 3D FULL: step + reconstruction
         cur ^= 1;
     }
+    return launch_advance_time(g->t_dev, nsteps, dt, g->stream);
+}
+
+// A run on a small 2D grid: coefficients, one cluster launch, clock.
+cudaError_t issue_small(gals_grid *g, const VelParams &vp, int trace, double dt, int nsteps, bool first_explicit,
+                        int64_t &launches)
+{
+    launches = (vp.kind == VK_WAVES2D ? 2 : 1) + 2;
+    cudaError_t ce = launch_coef_table(g->coef, vp, g->t_dev, dt, nsteps, g->stream);
+    if (ce != cudaSuccess) return ce;
+    const StepLaunch a = step_launch(g, vp, trace, dt, 0, g->cur, first_explicit);
+    SmallLaunch r{};
+    r.in = a.in;
+    r.out = g->buf[g->cur ^ (nsteps & 1)];
+    r.geom = a.geom;
+    r.vp = vp;
+    r.coef = g->coef;
+    r.dt = dt;
+    r.trace = a.trace;
+    r.cell = a.cross_in == CROSS_CELL;
+    r.planes = a.cross_in == CROSS_PLANE;
+    r.write_cross = a.write_cross;
+    r.nsteps = nsteps;
+    if ((ce = launch_step2d_small(r, g->stream)) != cudaSuccess) return ce;
     return launch_advance_time(g->t_dev, nsteps, dt, g->stream);
 }
 
@@ -680,6 +712,15 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
             int64_t nl = 0;
             if ((ce = issue_steps(g, vp, v->trace, dt, 1, fe_c, nl, &ip, &chk)) != cudaSuccess) {
                 what = "step launch";
+                return ce;
+            }
+            total += nl;
+            return cudaSuccess;
+        }
+        if (use_small(g, v->trace, cs)) {
+            int64_t nl = 0;
+            if ((ce = issue_small(g, vp, v->trace, dt, cs, fe_c, nl)) != cudaSuccess) {
+                what = "small-grid launch";
                 return ce;
             }
             total += nl;

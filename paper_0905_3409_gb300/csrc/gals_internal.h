@@ -49,6 +49,32 @@ int run2d_tiles(const Geom &g);
 int run2d_max_cells(int axis);
 cudaError_t launch_step2d_run(const RunLaunch &a, cudaStream_t s);
 
+// A run of steps on a small 2D grid in one launch of one cluster (step2d_small.cu).  Rule
+// (small2d_fits): at most kSmallNodes nodes in rows of at most kSmallColumns, and the
+// blocks' shared memory; a run of at least kSmallSteps steps.  At every size up to the limit
+// it is the faster way (128 x 96: 1.8 us per step against 7.2 for the banded launches;
+// 512 x 24: 2.4 against 6.7); larger grids keep the launches per step and band that
+// gals_last_step_launches is specified to count, and a run of fewer than 8 steps gains
+// little, its coefficient and clock kernels being most of it (5.3 us per step at 8 steps
+// against 9.9 at 7 of a first launch per step).
+constexpr int kSmallNodes = 12288, kSmallColumns = 512, kSmallSteps = 8;
+constexpr int kSmallMaxBytes = 96 * 1024;
+struct SmallLaunch {
+    const float *in;       // state at the run's start (all planes)
+    float *out;            // state at its end; may be `in`
+    Geom geom;
+    VelParams vp;
+    const StageCoef *coef; // stage coefficients of the run's steps
+    double dt;
+    int trace;             // TR_EULER / TR_RK3 / TR_HEUN
+    int cell;              // approach B
+    int planes;            // the first step reads the stored mixed derivatives
+    int write_cross;       // write the mixed-derivative plane of the end state
+    int nsteps;
+};
+bool small2d_fits(const Geom &g);
+cudaError_t launch_step2d_small(const SmallLaunch &a, cudaStream_t s);
+
 // Granularity of StepLaunch bands: the 2D tile height, the 3D tile depth.
 int band_unit(int dim);
 

@@ -141,12 +141,17 @@ __device__ __forceinline__ Sep2 sep_factors2(F2 s)
 // folded in: u = ku Ay, v = kv Sy, du/dx = k00 Ay, du/dy = k01 By, dv/dx = k10 Sy.
 struct VCol { float ku, kv, k00, k01, k10; };
 
+__device__ __forceinline__ VCol vortex_col_from(float A, float B, float c)
+{
+    const float S = __fmaf_rn(B, 0.5f, 0.5f), cp = c * kPi;
+    return VCol{c * S, -c * A, -cp * A, (2.f * cp) * S, (-2.f * cp) * B};
+}
+
 __device__ __forceinline__ VCol vortex_col(float x, float c)
 {
     float A, B;
     sincos_turn(x, &A, &B);
-    const float S = __fmaf_rn(B, 0.5f, 0.5f), cp = c * kPi;
-    return VCol{c * S, -c * A, -cp * A, (2.f * cp) * S, (-2.f * cp) * B};
+    return vortex_col_from(A, B, c);
 }
 
 // v(x, t+dt) at two nodes of one column; the single vortex uses the column factors cx
@@ -244,6 +249,46 @@ __device__ __forceinline__ void gather_lane(const float *__restrict__ in, const 
     if (CR == CROSS_CELL) cross_cell2d(c, g.ih0, g.ih1);
 }
 
+// The update of two nodes from their traced feet: cell location, gather(k, l, c) of each
+// lane's cell data, Hermite value and gradient, psi+ = J^T grad H (or Heun's method).
+template <int TR, int VK, class Gather>
+__device__ __forceinline__ void node2d_foot(const Geom &g, const VelParams &vp, const StageCoef &sc,
+                                            const StageCoefPair *scp, float dt, int i0, int j0, int i1,
+                                            int j1, F2 x, F2 y, F2 dx, F2 dy, const F2 J[4],
+                                            const VCol &cx, const Sep2 &ry, Gather gather, F2 &phi,
+                                            F2 &px, F2 &py, const V2p *a1)
+{
+    int k0, l0, k1, l1;
+    F2 xi, eta;
+    locate_pair(i0, i1, mul2(dx, bc(g.ih0)), g.n0, k0, k1, xi);
+    locate_pair(j0, j1, mul2(dy, bc(g.ih1)), g.n1, l0, l1, eta);
+
+    float c0[4][4], c1[4][4];
+    gather(k0, l0, c0);
+    gather(k1, l1, c1);
+    F2 c[4][4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) c[v][a] = make_float2(c0[v][a], c1[v][a]);
+
+    const Basis2 bx = basis_pair(xi, g.h0, g.ih0);
+    const Basis2 by = basis_pair(eta, g.h1, g.ih1);
+    F2 H, Hx, Hy;
+    hermite2d_pair(c, bx, by, H, Hx, Hy);
+    phi = H;
+    if (TR == TR_HEUN) {
+        // CIR gradient update (Sec. 4): Dv at the foot at time t (stage coefficients 1),
+        // Dv at the node at t + dt (the trace's first stage, evaluated again)
+        const V2p Df = vel2d_pair<VK>(vp, sc, scp, 1, add2(x, dx), add2(y, dy));
+        const V2p Dn = (VK == VK_FOURIER2D && a1 != nullptr) ? *a1 : stage1_pair<VK>(vp, sc, scp, x, y, cx, ry);
+        heun_psi2(Df, Dn, dt, Hx, Hy, px, py);
+        return;
+    }
+    px = fma2(J[0], Hx, mul2(J[2], Hy));  // (J^T grad H)_x
+    py = fma2(J[1], Hx, mul2(J[3], Hy));  // (J^T grad H)_y
+}
+
 // Update of two nodes (i0, j0) and (i1, j1): phi+, psi_x+, psi_y+ per lane; the staged
 // tile (W columns from column x0 - HX; SX: from column x0) has HYV halo rows.
 template <int TY, int TR, int VK, int CR, int HYV = HY, bool COH = false, int W = TW, bool SX = false>
@@ -271,36 +316,10 @@ __device__ __forceinline__ void node2d_pair(const float *__restrict__ in, const 
         trace2d_pair<TR, VK>(stage1_pair<VK>(vp, sc, scp, x, y, cx, ry), vp, sc, scp, x, y, dt, dx,
                              dy, J);
     }
-    (void)J;
-    int k0, l0, k1, l1;
-    F2 xi, eta;
-    locate_pair(i0, i1, mul2(dx, bc(g.ih0)), g.n0, k0, k1, xi);
-    locate_pair(j0, j1, mul2(dy, bc(g.ih1)), g.n1, l0, l1, eta);
-
-    float c0[4][4], c1[4][4];
-    gather_lane<TY, CR, HYV, COH, W, SX>(in, g, tile, x0, y0, k0, l0, c0);
-    gather_lane<TY, CR, HYV, COH, W, SX>(in, g, tile, x0, y0, k1, l1, c1);
-    F2 c[4][4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) c[v][a] = make_float2(c0[v][a], c1[v][a]);
-
-    const Basis2 bx = basis_pair(xi, g.h0, g.ih0);
-    const Basis2 by = basis_pair(eta, g.h1, g.ih1);
-    F2 H, Hx, Hy;
-    hermite2d_pair(c, bx, by, H, Hx, Hy);
-    phi = H;
-    if (TR == TR_HEUN) {
-        // CIR gradient update (Sec. 4): Dv at the foot at time t (stage coefficients 1),
-        // Dv at the node at t + dt (the trace's first stage, evaluated again)
-        const V2p Df = vel2d_pair<VK>(vp, sc, scp, 1, add2(x, dx), add2(y, dy));
-        const V2p Dn = (VK == VK_FOURIER2D && a1 != nullptr) ? *a1 : stage1_pair<VK>(vp, sc, scp, x, y, cx, ry);
-        heun_psi2(Df, Dn, dt, Hx, Hy, px, py);
-        return;
-    }
-    px = fma2(J[0], Hx, mul2(J[2], Hy));  // (J^T grad H)_x
-    py = fma2(J[1], Hx, mul2(J[3], Hy));  // (J^T grad H)_y
+    node2d_foot<TR, VK>(g, vp, sc, scp, dt, i0, j0, i1, j1, x, y, dx, dy, J, cx, ry,
+                        [&](int k, int l, float c[4][4]) {
+                            gather_lane<TY, CR, HYV, COH, W, SX>(in, g, tile, x0, y0, k, l, c);
+                        }, phi, px, py, a1);
 }
 
 // One tile step: origin (x0, y0).  `tile` is the dynamic shared buffer for the staged
