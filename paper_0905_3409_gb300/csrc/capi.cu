@@ -64,8 +64,9 @@ struct gals_grid {
     double t = 0.0;
     int64_t steps = 0;
     double *t_dev = nullptr;
-    CUtensorMap maps[2][3];       // TMA maps per buffer: [b][0] COMPACT box, [b][1] FULL box,
-                                  // [b][2] 3D reconstruction box
+    // TMA maps per buffer: [b][0] phi and psi, [b][1] all planes; [b][2] 3D reconstruction box,
+    // 2D short tiles: [b][2] phi and psi, [b][3] all planes
+    CUtensorMap maps[2][4];
     float *trace_buf = nullptr;   // surrogate trace of the current step: dx, dy, J (6 planes)
     char *pt_buf = nullptr;       // gals_eval_points: device staging of host points / results
     size_t pt_cap = 0;
@@ -149,8 +150,14 @@ gals_status make_velparams(gals_grid *g, const gals_velocity *v, VelParams &vp)
     return GALS_OK;
 }
 
-// Kernel launch descriptor of step s of a call, from buffer cur to buffer cur ^ 1.
-StepLaunch step_launch(gals_grid *g, const VelParams &vp, int trace, double dt, int s, int cur,
+// Kernel launch descriptor of step s of a run of nsteps, from buffer cur to buffer cur ^ 1.
+// Between the steps of a run nobody reads the mixed derivatives of approach A but the next
+// step, so only the run's first step reads their stored planes and only its last one
+// writes them; the steps between rebuild them from the gradients around each cell (the
+// COMPACT layout's way, the same stencils and bits).  In 2D that moves 24 instead of 32
+// bytes per node and leaves out the exchange of psi_y+ at the end of a tile: 4096^2 vortex
+// 119.4 us per step against 128.5 (107.8 with the walked tiles of step2d_walk.cuh).
+StepLaunch step_launch(gals_grid *g, const VelParams &vp, int trace, double dt, int s, int nsteps, int cur,
                        bool first_explicit)
 {
     StepLaunch a{};
@@ -160,8 +167,7 @@ StepLaunch step_launch(gals_grid *g, const VelParams &vp, int trace, double dt, 
     a.vp = vp;
     a.coef = g->coef + s;
     a.dt = dt;
-    a.tmap3 = &g->maps[cur][0];
-    a.tmap4 = &g->maps[cur][1];
+    for (int k = 0; k < 4; ++k) a.tmap[k >> 1][k & 1] = &g->maps[cur][k];
     a.tmap_cross = &g->maps[cur ^ 1][2];
     a.err = g->err_dev;
     a.trace = trace == GALS_TRACE_EULER      ? TR_EULER
@@ -172,8 +178,8 @@ StepLaunch step_launch(gals_grid *g, const VelParams &vp, int trace, double dt, 
         a.cross_in = CROSS_CELL;  // approach B: mixed derivatives per cell, none stored
         a.write_cross = 0;
     } else if (g->layout == GALS_LAYOUT_FULL) {
-        a.cross_in = CROSS_PLANE;
-        a.write_cross = 1;
+        a.cross_in = (s == 0 || g->dim == 3) ? CROSS_PLANE : CROSS_RECON;
+        a.write_cross = s == nsteps - 1 || g->dim == 3;
     } else {
         a.cross_in = (s == 0 && first_explicit) ? CROSS_PLANE : CROSS_RECON;
         a.write_cross = 0;
@@ -277,7 +283,7 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
                     if (b > 0 && (ce = cudaStreamWaitEvent(bs, prev[b - 1], 0)) != cudaSuccess) return ce;
                     if (b + 1 < nb && (ce = cudaStreamWaitEvent(bs, prev[b + 1], 0)) != cudaSuccess) return ce;
                 }
-                StepLaunch a = step_launch(g, vp, trace, dt, s, cur, first_explicit);
+                StepLaunch a = step_launch(g, vp, trace, dt, s, nsteps, cur, first_explicit);
                 a.band_lo = bands->row[b];
                 a.band_hi = bands->row[b + 1];
                 if ((ce = launch_step2d(a, bs)) != cudaSuccess) return ce;
@@ -296,7 +302,7 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
         const int tiles = run2d_tiles(g->geom);
         const int chunk = (int)((INT32_MAX - (1 << 20)) / tiles);
         for (int s0 = 0; s0 < nsteps; s0 += chunk) {
-            StepLaunch a = step_launch(g, vp, trace, dt, 0, cur, first_explicit);
+            StepLaunch a = step_launch(g, vp, trace, dt, 0, 1, cur, first_explicit);
             RunLaunch r{};
             r.buf[0] = g->buf[0];
             r.buf[1] = g->buf[1];
@@ -320,7 +326,7 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
         return launch_advance_time(g->t_dev, nsteps, dt, g->stream);
     }
     for (int s = 0; s < nsteps; ++s) {
-        StepLaunch a = step_launch(g, vp, trace, dt, s, cur, first_explicit);
+        StepLaunch a = step_launch(g, vp, trace, dt, s, nsteps, cur, first_explicit);
         if (trace == GALS_TRACE_SURROGATE) {
             // learned trace of this step (with RK3 fallback per tile), then the Hermite stage
             ce = mlp::launch_mlp_trace(*ip, g->geom, vp, g->coef + s, g->t_dev, s, dt, g->trace_buf,
@@ -345,7 +351,7 @@ cudaError_t issue_small(gals_grid *g, const VelParams &vp, int trace, double dt,
     launches = (vp.kind == VK_WAVES2D ? 2 : 1) + 2;
     cudaError_t ce = launch_coef_table(g->coef, vp, g->t_dev, dt, nsteps, g->stream);
     if (ce != cudaSuccess) return ce;
-    const StepLaunch a = step_launch(g, vp, trace, dt, 0, g->cur, first_explicit);
+    const StepLaunch a = step_launch(g, vp, trace, dt, 0, 1, g->cur, first_explicit);
     SmallLaunch r{};
     r.in = a.in;
     r.out = g->buf[g->cur ^ (nsteps & 1)];
@@ -501,13 +507,13 @@ gals_status gals_create_grid(const gals_grid_desc *d, gals_grid **out)
     // TMA maps of each buffer with the step kernels' tile boxes:
     // 2D (x, y, plane), 3D (x, y, z, plane); 3D also the reconstruction kernel's box
     for (int b = 0; b < 2; ++b)
-        for (int v = 0; v < (g->dim == 2 ? 2 : 3); ++v) {
+        for (int v = 0; v < (g->dim == 2 ? 4 : 3); ++v) {
             if (g->dim == 2) {
-                const int np = v == 0 ? 3 : 4;
+                const int np = 3 + (v & 1);
                 const uint64_t dims[3] = {(uint64_t)G.n0, (uint64_t)G.n1, (uint64_t)np};
                 const uint64_t strides[2] = {(uint64_t)G.pitch * 4, (uint64_t)G.plane * 4};
                 uint32_t box[3];
-                tile_box2d(np, box);
+                tile_box2d(v >> 1, np, box);
                 e = make_tile_map(&g->maps[b][v], g->buf[b], 3, dims, strides, box);
             } else {
                 uint32_t box[4];
@@ -930,7 +936,7 @@ static gals_status step_host_impl(gals_grid *g, const gals_velocity *v, double d
                                   nr, cudaMemcpyHostToDevice, g->hs_in);
         if (e == cudaSuccess) e = cudaEventRecord(g->hs_in_ev[b], g->hs_in);
     };
-    StepLaunch a = step_launch(g, vp, v->trace, dt, 0, cur, false);
+    StepLaunch a = step_launch(g, vp, v->trace, dt, 0, 1, cur, false);
     auto step_out = [&](int b) {
         if ((e = cudaStreamWaitEvent(g->stream, g->hs_in_ev[std::min(nb - 1, b + K)], 0)) != cudaSuccess) return;
         a.band_lo = b * R;

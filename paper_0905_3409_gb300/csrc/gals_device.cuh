@@ -37,7 +37,8 @@ enum TraceKind { TR_EULER = 0, TR_RK3 = 1, TR_GIVEN = 2, TR_HEUN = 3 };
 // Where a cell's mixed derivatives come from: the stored planes (approach A, FULL), the
 // psi windows around the cell (approach A, COMPACT), or the cell's own gradients
 // (approach B of Sec. 2.3).
-enum CrossSrc { CROSS_PLANE = 0, CROSS_RECON = 1, CROSS_CELL = 2 };
+// NONE: phi and psi only (the caller derives the mixed derivatives).
+enum CrossSrc { CROSS_PLANE = 0, CROSS_RECON = 1, CROSS_CELL = 2, CROSS_NONE = 3 };
 
 // Velocity descriptor as passed to kernels (by value).
 struct VelParams {
@@ -118,6 +119,10 @@ __device__ __forceinline__ int64_t plane_extent(const Geom &g)
 {
     return (int64_t)g.n2 * g.n1 * g.pitch;
 }
+
+// Coordinate of node i: one rounding wherever it is computed (left to the compiler, the
+// multiply and the add were fused in some kernels and not in others).
+__device__ __forceinline__ float node_pos(float lo, int i, float h) { return __fmaf_rn((float)i, h, lo); }
 
 // Time-dependent scalars of the three RK3 stage times (t+dt, t, t+dt/2) of one step.
 // A table of these (one entry per step of a gals_step call) is filled once per call by
@@ -500,15 +505,15 @@ __device__ __forceinline__ void hermite3d(const float c[8][8], const Basis1 &bx,
 __device__ __forceinline__ float cell_vertex(float e0, float e1, float f0, float f1, int u, int w)
 {
     const float ne = u ? e1 : e0, fe = u ? e0 : e1, nf = w ? f1 : f0, ff = w ? f0 : f1;
-    return 0.75f * (ne + nf) - 0.25f * (fe + ff);
+    return __fmaf_rn(0.75f, __fadd_rn(ne, nf), -0.25f * __fadd_rn(fe, ff));
 }
 
 // 2D cell, c[v][a] (v = vx + 2 vy; a = 0 phi, 1 phi_x, 2 phi_y, 3 phi_xy): phi_xy at the
 // four vertices from psi_x differenced along y and psi_y differenced along x.
 __device__ __forceinline__ void cross_cell2d(float c[4][4], float ih0, float ih1)
 {
-    const float e0 = (c[2][1] - c[0][1]) * ih1, e1 = (c[3][1] - c[1][1]) * ih1;
-    const float f0 = (c[1][2] - c[0][2]) * ih0, f1 = (c[3][2] - c[2][2]) * ih0;
+    const float e0 = __fmul_rn(c[2][1] - c[0][1], ih1), e1 = __fmul_rn(c[3][1] - c[1][1], ih1);
+    const float f0 = __fmul_rn(c[1][2] - c[0][2], ih0), f1 = __fmul_rn(c[3][2] - c[2][2], ih0);
 #pragma unroll
     for (int v = 0; v < 4; ++v) c[v][3] = cell_vertex(e0, e1, f0, f1, v & 1, v >> 1);
 }

@@ -19,8 +19,9 @@ struct StepLaunch {
     int trace;           // TR_EULER / TR_RK3
     int cross_in;        // CROSS_PLANE: read mixed derivatives; CROSS_RECON: rebuild from psi
     int write_cross;     // 1: also write the mixed-derivative planes of the new state
-    const CUtensorMap *tmap4; // TMA map of `in` for reading stored mixed derivatives
-    const CUtensorMap *tmap3; // TMA map of `in` for rebuilding them (COMPACT)
+    // TMA maps of `in`, [short 2D tiles][4 or (3D: 8) planes with the stored mixed derivatives:
+    // 1, phi and psi only: 0]
+    const CUtensorMap *tmap[2][2];
     const CUtensorMap *tmap_cross; // 3D FULL: TMA map of `out` with the reconstruction box
     int *err;            // device error word (kErrTmaTimeout on a lost tile copy)
     // the band of nodes to update along the last axis (2D rows, 3D z-levels), [lo, hi);
@@ -78,8 +79,8 @@ cudaError_t launch_step2d_small(const SmallLaunch &a, cudaStream_t s);
 // Granularity of StepLaunch bands: the 2D tile height, the 3D tile depth.
 int band_unit(int dim);
 
-// Box of the 2D step kernel's staged tile for np planes; its output rows per block.
-void tile_box2d(int np, uint32_t box[3]);
+// Box of the 2D step kernels' staged tile (tall or short) for np planes; rows of a tall tile.
+void tile_box2d(int is_short, int np, uint32_t box[3]);
 int tile_rows2d();
 // Box (x, y, z, planes) of the 3D step kernel's staged tile.
 void tile_box3d(int cross_recon, uint32_t box[4]);

@@ -18,6 +18,7 @@ namespace gals {
 typedef float2 F2;
 
 __device__ __forceinline__ F2 bc(float a) { return make_float2(a, a); }
+// (the compiler fuses a mul2 into an add2: not for sums of products, see vel2d_pair)
 __device__ __forceinline__ F2 add2(F2 a, F2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ F2 mul2(F2 a, F2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) { return __ffma2_rn(a, b, c); }
@@ -54,18 +55,24 @@ struct StageCoefPair {
     F2 A[3][16], Al[3][16], All[3][16];
 };
 
-template <int VK>
+// v and Dv at two points.  SUM: r.u, r.v are the velocity added to (u0, v0), the last product
+// and the addition in one rounding: the trace needs only the sum of its first two stages.
+// (A product and an addition written apart are fused by the compiler where it sees fit, so
+// two kernels could round the same node differently.)
+template <int VK, bool SUM = false>
 __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &sc,
-                                          const StageCoefPair *scp, int stage, F2 x, F2 y)
+                                          const StageCoefPair *scp, int stage, F2 x, F2 y,
+                                          F2 u0 = make_float2(0.f, 0.f), F2 v0 = make_float2(0.f, 0.f))
 {
+    auto prod = [](F2 p, F2 q, F2 acc) { return SUM ? fma2(p, q, acc) : mul2(p, q); };
     V2p r;
     if (VK == VK_CONST) {
-        r.u = bc(vp.c0); r.v = bc(vp.c1);
+        r.u = prod(bc(vp.c0), bc(1.f), u0); r.v = prod(bc(vp.c1), bc(1.f), v0);
         r.d00 = r.d01 = r.d10 = r.d11 = bc(0.f);
     } else if (VK == VK_ROTATION) {
         const F2 w = bc(vp.omega);
-        r.u = mul2(bc(-vp.omega), sub2(y, bc(vp.cy)));
-        r.v = mul2(w, sub2(x, bc(vp.cx)));
+        r.u = prod(bc(-vp.omega), sub2(y, bc(vp.cy)), u0);
+        r.v = prod(w, sub2(x, bc(vp.cx)), v0);
         r.d00 = bc(0.f); r.d01 = bc(-vp.omega); r.d10 = w; r.d11 = bc(0.f);
     } else if (VK == VK_VORTEX2D) {
         // u = -c sin^2(pi x) sin(2 pi y), v = c sin(2 pi x) sin^2(pi y) in the factors
@@ -75,8 +82,8 @@ __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &
         sincos_turn2(y, Ay, By);
         const float c = sc.mod[stage], h = 0.5f * c;
         const F2 cSx = fma2(Bx, bc(h), bc(h)), mcSy = fma2(By, bc(-h), bc(-h));
-        r.u = mul2(cSx, Ay);
-        r.v = mul2(Ax, mcSy);
+        r.u = prod(cSx, Ay, u0);
+        r.v = prod(Ax, mcSy, v0);
         r.d00 = mul2(bc(-c * kPi), mul2(Ax, Ay));
         r.d01 = mul2(bc(2.f * kPi), mul2(cSx, By));
         r.d10 = mul2(bc(2.f * kPi), mul2(Bx, mcSy));
@@ -84,7 +91,7 @@ __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &
     } else if (VK == VK_PSEUDO1D) {
         const F2 arg = fma2(bc(vp.d0), x, mul2(bc(vp.d1), y));
         const F2 e = make_float2(__expf(arg.x), __expf(arg.y));
-        r.u = mul2(e, bc(vp.d0)); r.v = mul2(e, bc(vp.d1));
+        r.u = prod(e, bc(vp.d0), u0); r.v = prod(e, bc(vp.d1), v0);
         r.d00 = mul2(e, bc(vp.d0 * vp.d0)); r.d01 = mul2(e, bc(vp.d0 * vp.d1));
         r.d10 = r.d01; r.d11 = mul2(e, bc(vp.d1 * vp.d1));
     } else if (VK == VK_WAVES2D) {
@@ -107,7 +114,7 @@ __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &
             d01 = fma2(bc(q.y), cn, d01);
             d10 = fma2(bc(-q.x), cn, d10);
         }
-        r.u = u; r.v = v; r.d00 = d00; r.d01 = d01; r.d10 = d10; r.d11 = neg2(d00);
+        r.u = SUM ? fma2(u, bc(1.f), u0) : u; r.v = SUM ? fma2(v, bc(1.f), v0) : v; r.d00 = d00; r.d01 = d01; r.d10 = d10; r.d11 = neg2(d00);
     } else {  // VK_FOURIER2D: Psi = sum A_kl s_k(x) s_l(y), u = -Psi_y, v = Psi_x
         F2 s[5], c[5], sy_[5], cy_[5];
         sincospi2(x, s[1], c[1]);
@@ -137,7 +144,7 @@ __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &
             d01 = fma2(s[k], W, d01);
             d10 = fma2(mul2(bc(-kp * kp), s[k]), Vx, d10);
         }
-        r.u = u; r.v = v; r.d00 = d00; r.d01 = d01; r.d10 = d10; r.d11 = neg2(d00);
+        r.u = SUM ? fma2(u, bc(1.f), u0) : u; r.v = SUM ? fma2(v, bc(1.f), v0) : v; r.d00 = d00; r.d01 = d01; r.d10 = d10; r.d11 = neg2(d00);
     }
     return r;
 }
@@ -153,8 +160,8 @@ __device__ __forceinline__ void heun_psi2(const V2p &Df, const V2p &Dn, float dt
     const F2 sx = fma2(bc(dt), k1x, gx), sy = fma2(bc(dt), k1y, gy);
     const F2 k2x = neg2(fma2(Dn.d00, sx, mul2(Dn.d10, sy)));
     const F2 k2y = neg2(fma2(Dn.d01, sx, mul2(Dn.d11, sy)));
-    px = fma2(bc(0.5f * dt), add2(k1x, k2x), gx);
-    py = fma2(bc(0.5f * dt), add2(k1y, k2y), gy);
+    px = fma2(bc(0.5f * dt), fma2(k1x, bc(1.f), k2x), gx);
+    py = fma2(bc(0.5f * dt), fma2(k1y, bc(1.f), k2y), gy);
 }
 
 // Superconsistent trace of Sec. 5.1 for two nodes; a = v(x, t+dt) supplied by the caller.
@@ -173,7 +180,8 @@ __device__ __forceinline__ void trace2d_pair(const V2p &a, const VelParams &vp,
     // stage 1: x1 = x - dt v1, J1 = I - dt Dv1
     const F2 J1_00 = fma2(mdt, a.d00, one), J1_01 = mul2(mdt, a.d01);
     const F2 J1_10 = mul2(mdt, a.d10), J1_11 = fma2(mdt, a.d11, one);
-    const V2p b = vel2d_pair<VK>(vp, sc, scp, 1, fma2(mdt, a.u, x), fma2(mdt, a.v, y));
+    // b: Dv2, and v1 + v2
+    const V2p b = vel2d_pair<VK, true>(vp, sc, scp, 1, fma2(mdt, a.u, x), fma2(mdt, a.v, y), a.u, a.v);
     // S = Dv1 + Dv2 J1 (Dv1 is the accumulator of the product)
     const F2 S00 = fma2(b.d00, J1_00, fma2(b.d01, J1_10, a.d00));
     const F2 S01 = fma2(b.d00, J1_01, fma2(b.d01, J1_11, a.d01));
@@ -182,13 +190,12 @@ __device__ __forceinline__ void trace2d_pair(const V2p &a, const VelParams &vp,
     // stage 2: x2 = x - dt (v1 + v2)/4, J2 = I - dt S / 4, kept as G = (-2 dt / 3) J2
     const F2 mq = bc(-0.25f * dt), m23 = bc(-2.f * dt / 3.f), kq = bc((-2.f * dt / 3.f) * (-0.25f * dt));
     const F2 G00 = fma2(kq, S00, m23), G01 = mul2(kq, S01), G10 = mul2(kq, S10), G11 = fma2(kq, S11, m23);
-    const V2p c = vel2d_pair<VK>(vp, sc, scp, 2, fma2(mq, add2(a.u, b.u), x),
-                                 fma2(mq, add2(a.v, b.v), y));
+    const V2p c = vel2d_pair<VK>(vp, sc, scp, 2, fma2(mq, b.u, x), fma2(mq, b.v, y));
     // foot = x - dt (w3 + (w1 + w2 - 2 w3)/6): exact for constant v;
     // J = I - dt S / 6 - 2 dt Dv3 J2 / 3 = (I - dt S / 6) + Dv3 G (= I when Dv = 0)
     const F2 i6 = bc(1.f / 6.f), m2 = bc(-2.f), m6 = bc(-dt / 6.f);
-    dx = mul2(mdt, fma2(fma2(m2, c.u, add2(a.u, b.u)), i6, c.u));
-    dy = mul2(mdt, fma2(fma2(m2, c.v, add2(a.v, b.v)), i6, c.v));
+    dx = mul2(mdt, fma2(fma2(m2, c.u, b.u), i6, c.u));
+    dy = mul2(mdt, fma2(fma2(m2, c.v, b.v), i6, c.v));
     J[0] = fma2(c.d00, G00, fma2(c.d01, G10, fma2(m6, S00, one)));
     J[1] = fma2(c.d00, G01, fma2(c.d01, G11, mul2(m6, S01)));
     J[2] = fma2(c.d10, G00, fma2(c.d11, G10, mul2(m6, S10)));
@@ -276,6 +283,23 @@ __device__ __forceinline__ void hermite2d_pair(const F2 c[4][4], const Basis2 &b
     Hx = hval2(by, Pd0, Pd1, Qd0, Qd1);
 }
 
+// Approach B for the cells of both lanes (the scalar cross_cell2d, lane by lane).
+__device__ __forceinline__ void cross_cell2d_pair(F2 c[4][4], float ih0, float ih1)
+{
+    float a[4][4], b[4][4];
+#pragma unroll
+    for (int v = 0; v < 4; ++v)
+#pragma unroll
+        for (int p = 0; p < 3; ++p) {
+            a[v][p] = c[v][p].x;
+            b[v][p] = c[v][p].y;
+        }
+    cross_cell2d(a, ih0, ih1);
+    cross_cell2d(b, ih0, ih1);
+#pragma unroll
+    for (int v = 0; v < 4; ++v) c[v][3] = make_float2(a[v][3], b[v][3]);
+}
+
 // ---------------------------------------------------------------- 3D, two nodes per thread
 
 struct V3p { F2 v[3]; F2 d[9]; };
@@ -283,13 +307,14 @@ struct V3p { F2 v[3]; F2 d[9]; };
 // The deformation field from its folded xy products P1 = 2 Sx Ay, P2 = -Ax Sy,
 // P3 = -Ax Ay, P4 = 4 pi Sx By, P5 = -2 pi Bx Sy, P6 = -2 pi Bx Ay, P7 = -2 pi Ax By and
 // z factors Azc = c Az, Szc = c Sz, Bzc = 2 pi c Bz (see vel3d_pair).
+template <bool SUM = false>
 __device__ __forceinline__ void deform_terms(F2 P1, F2 P2, F2 P3, F2 P4, F2 P5, F2 P6, F2 P7,
-                                             F2 Azc, F2 Szc, F2 Bzc, V3p &r)
+                                             F2 Azc, F2 Szc, F2 Bzc, V3p &r, const F2 *v0 = nullptr)
 {
     const F2 T = mul2(P3, Azc);                  // -c Ax Ay Az
-    r.v[0] = mul2(P1, Azc);
-    r.v[1] = mul2(P2, Azc);
-    r.v[2] = mul2(P3, Szc);
+    r.v[0] = SUM ? fma2(P1, Azc, v0[0]) : mul2(P1, Azc);
+    r.v[1] = SUM ? fma2(P2, Azc, v0[1]) : mul2(P2, Azc);
+    r.v[2] = SUM ? fma2(P3, Szc, v0[2]) : mul2(P3, Szc);
     r.d[0] = mul2(bc(2.f * kPi), T);
     r.d[1] = mul2(P4, Azc);
     r.d[2] = mul2(P1, Bzc);
@@ -304,19 +329,23 @@ __device__ __forceinline__ void deform_terms(F2 P1, F2 P2, F2 P3, F2 P4, F2 P5, 
 // v and Dv (Dv[3i+j] = dv_i/dx_j) at two points; DEFORM3D is LeVeque's field
 // u = 2 sin^2(pi x) sin(2 pi y) sin(2 pi z) c, v = -sin(2 pi x) sin^2(pi y) sin(2 pi z) c,
 // w = -sin(2 pi x) sin(2 pi y) sin^2(pi z) c with c = cos(pi t / T).
-template <int VK>
+// SUM: r.v is the velocity added to v0 (see vel2d_pair).
+template <int VK, bool SUM = false>
 __device__ __forceinline__ V3p vel3d_pair(const VelParams &vp, const StageCoef &sc, int stage,
-                                          F2 x, F2 y, F2 z)
+                                          F2 x, F2 y, F2 z, const F2 *v0 = nullptr)
 {
     V3p r;
 #pragma unroll
     for (int a = 0; a < 9; ++a) r.d[a] = bc(0.f);
     if (VK == VK_CONST) {
         r.v[0] = bc(vp.c0); r.v[1] = bc(vp.c1); r.v[2] = bc(vp.c2);
+        if (SUM)
+            for (int a = 0; a < 3; ++a) r.v[a] = fma2(r.v[a], bc(1.f), v0[a]);
     } else if (VK == VK_ROTATION) {
-        r.v[0] = mul2(bc(-vp.omega), sub2(y, bc(vp.cy)));
-        r.v[1] = mul2(bc(vp.omega), sub2(x, bc(vp.cx)));
-        r.v[2] = bc(0.f);
+        const F2 ry = sub2(y, bc(vp.cy)), rx = sub2(x, bc(vp.cx));
+        r.v[0] = SUM ? fma2(bc(-vp.omega), ry, v0[0]) : mul2(bc(-vp.omega), ry);
+        r.v[1] = SUM ? fma2(bc(vp.omega), rx, v0[1]) : mul2(bc(vp.omega), rx);
+        r.v[2] = SUM ? v0[2] : bc(0.f);
         r.d[1] = bc(-vp.omega); r.d[3] = bc(vp.omega);
     } else {  // VK_DEFORM3D
         // In the factors A = sin a, B = cos a of a = 2 pi (s - 1/2) and S = sin^2(pi s) =
@@ -331,8 +360,8 @@ __device__ __forceinline__ V3p vel3d_pair(const VelParams &vp, const StageCoef &
         const F2 Sx2 = add2(Bx, bc(1.f)), Bxm = mul2(bc(-2.f * kPi), Bx);
         const F2 Sy = fma2(By, bc(0.5f), bc(0.5f)), By2 = mul2(bc(2.f * kPi), By);
         const F2 Azc = mul2(bc(c), Az), Szc = fma2(Bz, bc(h), bc(h)), Bzc = mul2(bc(2.f * kPi * c), Bz);
-        deform_terms(mul2(Sx2, Ay), mul2(Axn, Sy), mul2(Axn, Ay), mul2(Sx2, By2), mul2(Bxm, Sy),
-                     mul2(Bxm, Ay), mul2(Axn, By2), Azc, Szc, Bzc, r);
+        deform_terms<SUM>(mul2(Sx2, Ay), mul2(Axn, Sy), mul2(Axn, Ay), mul2(Sx2, By2), mul2(Bxm, Sy),
+                          mul2(Bxm, Ay), mul2(Axn, By2), Azc, Szc, Bzc, r, v0);
     }
     return r;
 }
@@ -361,7 +390,7 @@ __device__ __forceinline__ void heun_psi3(const V3p &Df, const V3p &Dn, float dt
     for (int a = 0; a < 3; ++a)
         k2[a] = neg2(fma2(Dn.d[a], s[0], fma2(Dn.d[3 + a], s[1], mul2(Dn.d[6 + a], s[2]))));
 #pragma unroll
-    for (int a = 0; a < 3; ++a) psi[a] = fma2(bc(0.5f * dt), add2(k1[a], k2[a]), g[a]);
+    for (int a = 0; a < 3; ++a) psi[a] = fma2(bc(0.5f * dt), fma2(k1[a], bc(1.f), k2[a]), g[a]);
 }
 
 // Superconsistent RK3 trace of Sec. 5.1 for two nodes (a = v(x, t+dt) from the caller):
@@ -381,8 +410,9 @@ __device__ __forceinline__ void trace3d_pair(const V3p &a, const VelParams &vp, 
     F2 J1[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) J1[e] = (e % 4) == 0 ? fma2(mdt, a.d[e], one) : mul2(mdt, a.d[e]);
-    const V3p b = vel3d_pair<VK>(vp, sc, 1, fma2(mdt, a.v[0], x), fma2(mdt, a.v[1], y),
-                                 fma2(mdt, a.v[2], z));
+    // b: Dv2, and v1 + v2
+    const V3p b = vel3d_pair<VK, true>(vp, sc, 1, fma2(mdt, a.v[0], x), fma2(mdt, a.v[1], y),
+                                       fma2(mdt, a.v[2], z), a.v);
     // S = Dv1 + Dv2 J1 (Dv1 is the accumulator of the product)
     F2 S[9];
     matmul3_acc_pair(b.d, J1, a.d, S);
@@ -390,9 +420,7 @@ __device__ __forceinline__ void trace3d_pair(const V3p &a, const VelParams &vp, 
     F2 J2[9];
 #pragma unroll
     for (int e = 0; e < 9; ++e) J2[e] = (e % 4) == 0 ? fma2(mq, S[e], one) : mul2(mq, S[e]);
-    F2 s1[3];
-#pragma unroll
-    for (int i = 0; i < 3; ++i) s1[i] = add2(a.v[i], b.v[i]);
+    const F2 *s1 = b.v;
     const V3p c = vel3d_pair<VK>(vp, sc, 2, fma2(mq, s1[0], x), fma2(mq, s1[1], y), fma2(mq, s1[2], z));
     F2 N[9];
 #pragma unroll

@@ -109,8 +109,8 @@ template <int VK> struct SmallPair {
         r = r_;
         j0 = row0 + r;
         j1 = min(j0 + 1, g.n1 - 1);
-        x = bc(g.lo0 + (float)i * g.h0);
-        y = make_float2(g.lo1 + (float)j0 * g.h1, g.lo1 + (float)j1 * g.h1);
+        x = bc(node_pos(g.lo0, i, g.h0));
+        y = make_float2(node_pos(g.lo1, j0, g.h1), node_pos(g.lo1, j1, g.h1));
         if (VK == VK_VORTEX2D) {
             sincos_turn(x.x, &A, &B);
             ry = sep_factors2(y);

@@ -88,16 +88,16 @@ __device__ __forceinline__ void fourier_row(const StageCoef &sc, float y, int k,
     }
 }
 
-// v, Dv at the two nodes (rows r, r+1 of the tile) of a thread's column.
+// v, Dv at the two nodes (rows r, r1 of the tile) of a thread's column.
 template <int TY>
-__device__ __forceinline__ V2p fourier_stage1_pair(const FCol &f, const float (*fsum)[TY], int r)
+__device__ __forceinline__ V2p fourier_stage1_pair(const FCol &f, const float (*fsum)[TY], int r, int r1)
 {
     F2 u = bc(0.f), v = bc(0.f), d00 = bc(0.f), d01 = bc(0.f), d10 = bc(0.f);
 #pragma unroll
     for (int k = 1; k <= 4; ++k) {
-        const F2 Ux = make_float2(fsum[k - 1][r], fsum[k - 1][r + 1]);
-        const F2 Vx = make_float2(fsum[4 + k - 1][r], fsum[4 + k - 1][r + 1]);
-        const F2 W = make_float2(fsum[8 + k - 1][r], fsum[8 + k - 1][r + 1]);
+        const F2 Ux = make_float2(fsum[k - 1][r], fsum[k - 1][r1]);
+        const F2 Vx = make_float2(fsum[4 + k - 1][r], fsum[4 + k - 1][r1]);
+        const F2 W = make_float2(fsum[8 + k - 1][r], fsum[8 + k - 1][r1]);
         const float kp = (float)k * kPi;
         const F2 sk = bc(f.s[k]), ck = bc(f.c[k]);
         u = fma2(neg2(sk), Ux, u);
@@ -249,10 +249,10 @@ __device__ __forceinline__ void gather_lane(const float *__restrict__ in, const 
     if (CR == CROSS_CELL) cross_cell2d(c, g.ih0, g.ih1);
 }
 
-// The update of two nodes from their traced feet: cell location, gather(k, l, c) of each
-// lane's cell data, Hermite value and gradient, psi+ = J^T grad H (or Heun's method).
+// The update of two nodes from their traced feet: cell location, gather(k0, l0, k1, l1, c) of
+// the lanes' cell data, Hermite value and gradient, psi+ = J^T grad H (or Heun's method).
 template <int TR, int VK, class Gather>
-__device__ __forceinline__ void node2d_foot(const Geom &g, const VelParams &vp, const StageCoef &sc,
+__device__ __forceinline__ void node2d_feet(const Geom &g, const VelParams &vp, const StageCoef &sc,
                                             const StageCoefPair *scp, float dt, int i0, int j0, int i1,
                                             int j1, F2 x, F2 y, F2 dx, F2 dy, const F2 J[4],
                                             const VCol &cx, const Sep2 &ry, Gather gather, F2 &phi,
@@ -263,14 +263,8 @@ __device__ __forceinline__ void node2d_foot(const Geom &g, const VelParams &vp, 
     locate_pair(i0, i1, mul2(dx, bc(g.ih0)), g.n0, k0, k1, xi);
     locate_pair(j0, j1, mul2(dy, bc(g.ih1)), g.n1, l0, l1, eta);
 
-    float c0[4][4], c1[4][4];
-    gather(k0, l0, c0);
-    gather(k1, l1, c1);
     F2 c[4][4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v)
-#pragma unroll
-        for (int a = 0; a < 4; ++a) c[v][a] = make_float2(c0[v][a], c1[v][a]);
+    gather(k0, l0, k1, l1, c);
 
     const Basis2 bx = basis_pair(xi, g.h0, g.ih0);
     const Basis2 by = basis_pair(eta, g.h1, g.ih1);
@@ -280,13 +274,33 @@ __device__ __forceinline__ void node2d_foot(const Geom &g, const VelParams &vp, 
     if (TR == TR_HEUN) {
         // CIR gradient update (Sec. 4): Dv at the foot at time t (stage coefficients 1),
         // Dv at the node at t + dt (the trace's first stage, evaluated again)
-        const V2p Df = vel2d_pair<VK>(vp, sc, scp, 1, add2(x, dx), add2(y, dy));
+        const V2p Df = vel2d_pair<VK>(vp, sc, scp, 1, fma2(dx, bc(1.f), x), fma2(dy, bc(1.f), y));
         const V2p Dn = (VK == VK_FOURIER2D && a1 != nullptr) ? *a1 : stage1_pair<VK>(vp, sc, scp, x, y, cx, ry);
         heun_psi2(Df, Dn, dt, Hx, Hy, px, py);
         return;
     }
     px = fma2(J[0], Hx, mul2(J[2], Hy));  // (J^T grad H)_x
     py = fma2(J[1], Hx, mul2(J[3], Hy));  // (J^T grad H)_y
+}
+
+// The same with gather(k, l, c) of one lane's cell data.
+template <int TR, int VK, class Gather>
+__device__ __forceinline__ void node2d_foot(const Geom &g, const VelParams &vp, const StageCoef &sc,
+                                            const StageCoefPair *scp, float dt, int i0, int j0, int i1,
+                                            int j1, F2 x, F2 y, F2 dx, F2 dy, const F2 J[4],
+                                            const VCol &cx, const Sep2 &ry, Gather gather, F2 &phi,
+                                            F2 &px, F2 &py, const V2p *a1)
+{
+    node2d_feet<TR, VK>(g, vp, sc, scp, dt, i0, j0, i1, j1, x, y, dx, dy, J, cx, ry,
+                        [&](int k0, int l0, int k1, int l1, F2 c[4][4]) {
+                            float c0[4][4], c1[4][4];
+                            gather(k0, l0, c0);
+                            gather(k1, l1, c1);
+#pragma unroll
+                            for (int v = 0; v < 4; ++v)
+#pragma unroll
+                                for (int a = 0; a < 4; ++a) c[v][a] = make_float2(c0[v][a], c1[v][a]);
+                        }, phi, px, py, a1);
 }
 
 // Update of two nodes (i0, j0) and (i1, j1): phi+, psi_x+, psi_y+ per lane; the staged
@@ -396,7 +410,7 @@ __device__ __forceinline__ bool tile_step2d(const float *__restrict__ in, float 
         // stage-1 row sums of the tile's rows (rows past the grid repeat the last one)
         for (int e = tid; e < TY * 4; e += TX) {
             const int r = e >> 2, k = (e & 3) + 1;
-            const float yr = g.lo1 + (float)min(y0 + r, g.n1 - 1) * g.h1;
+            const float yr = node_pos(g.lo1, min(y0 + r, g.n1 - 1), g.h1);
             float ux, vx, w;
             fourier_row(sc, yr, k, ux, vx, w);
             sm.fsum[k - 1][r] = ux;
@@ -409,7 +423,7 @@ __device__ __forceinline__ bool tile_step2d(const float *__restrict__ in, float 
     const bool own = !OV || (tid >= 1 && tid <= TX - 2);  // a column of this tile's output
     constexpr int PQ = OV ? 1 : 2;                          // psy index of column i: i - x0 + 2
     const int rows = min(TY, g.n1 - y0);
-    const float xs = g.lo0 + (float)i * g.h0;
+    const float xs = node_pos(g.lo0, i, g.h0);
     const F2 x = bc(xs);
     const VCol cx = (VK == VK_VORTEX2D) ? vortex_col(xs, sc.mod[0]) : VCol{0.f, 0.f, 0.f, 0.f, 0.f};
     FCol fcol;
@@ -427,11 +441,11 @@ __device__ __forceinline__ bool tile_step2d(const float *__restrict__ in, float 
     if ((!OV || i >= 0) && i < g.n0) {
         for (int r = 0; r < rows; r += 2) {
             const int j0 = y0 + r, j1 = min(j0 + 1, g.n1 - 1);
-            const F2 y = make_float2(g.lo1 + (float)j0 * g.h1, g.lo1 + (float)j1 * g.h1);
+            const F2 y = make_float2(node_pos(g.lo1, j0, g.h1), node_pos(g.lo1, j1, g.h1));
             const Sep2 ry = (VK == VK_VORTEX2D) ? sep_factors2(y) : Sep2{bc(0.f), bc(0.f), bc(0.f)};
             F2 phi, px, py;
             if (VK == VK_FOURIER2D && TR != TR_GIVEN) {
-                const V2p a1 = fourier_stage1_pair<TY>(fcol, sm.fsum, r);
+                const V2p a1 = fourier_stage1_pair<TY>(fcol, sm.fsum, r, r + 1);
                 node2d_pair<TY, TR, VK, CR, HYV, COH, W, OV>(in, g, tile, gx0, y0, vp, sc, scp, dt, i, j0, i,
                                                    j1, x, y, cx, ry, phi, px, py, &a1);
             } else {
@@ -475,8 +489,8 @@ __device__ __forceinline__ bool tile_step2d(const float *__restrict__ in, float 
             const bool need = which == 0 ? (width == 1 && ih >= 0) : (!OV && ih >= 0 && ih < g.n0);
             if (!need) continue;
             const int r = 2 * rp, j0 = y0 + r, j1 = min(j0 + 1, g.n1 - 1);
-            const F2 xh = bc(g.lo0 + (float)ih * g.h0);
-            const F2 y = make_float2(g.lo1 + (float)j0 * g.h1, g.lo1 + (float)j1 * g.h1);
+            const F2 xh = bc(node_pos(g.lo0, ih, g.h0));
+            const F2 y = make_float2(node_pos(g.lo1, j0, g.h1), node_pos(g.lo1, j1, g.h1));
             const VCol cxh = (VK == VK_VORTEX2D) ? vortex_col(xh.x, sc.mod[0]) : VCol{0.f, 0.f, 0.f, 0.f, 0.f};
             const Sep2 ry = (VK == VK_VORTEX2D) ? sep_factors2(y) : Sep2{bc(0.f), bc(0.f), bc(0.f)};
             F2 phi, px, py;

@@ -161,7 +161,8 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
         F2 psi[3];
         if (TR == TR_HEUN) {
             // CIR gradient update (Sec. 4): Dv at the foot at time t, Dv at the node at t + dt
-            const V3p Df = vel3d_pair<VK>(vp, sc, 1, add2(X, d[0]), add2(Y, d[1]), add2(Z, d[2]));
+            const V3p Df = vel3d_pair<VK>(vp, sc, 1, fma2(d[0], bc(1.f), X), fma2(d[1], bc(1.f), Y),
+                                           fma2(d[2], bc(1.f), Z));
             const V3p Dn = stage1_pair<VK>(vp, sc, pre, X, Y, Z);
             heun_psi3(Df, Dn, dt, gr, psi);
         } else {
@@ -304,7 +305,7 @@ cudaError_t launch_t(const StepLaunch &a, cudaStream_t s, int zt0, int nzt)
     }
     dim3 block(TX, TY);
     dim3 grid((a.geom.n0 + TX - 1) / TX, (a.geom.n1 + TY - 1) / TY, nzt);
-    const CUtensorMap &map = CR == CROSS_PLANE ? *a.tmap4 : *a.tmap3;
+    const CUtensorMap &map = *a.tmap[0][CR == CROSS_PLANE];
     k_step3d<TR, VK, CR><<<grid, block, T::BYTES, s>>>(a.in, a.out, a.geom, a.vp, a.coef,
                                                       (float)a.dt, map, a.err, zt0);
     return cudaGetLastError();
