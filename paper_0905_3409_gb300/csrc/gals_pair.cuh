@@ -126,7 +126,8 @@ __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &
         sy_[2] = mul2(two, mul2(sy_[1], cy_[1]));          cy_[2] = fma2(mtwo, mul2(sy_[1], sy_[1]), one);
         sy_[3] = fma2(sy_[2], cy_[1], mul2(cy_[2], sy_[1])); cy_[3] = fma2(cy_[2], cy_[1], neg2(mul2(sy_[2], sy_[1])));
         sy_[4] = mul2(two, mul2(sy_[2], cy_[2]));          cy_[4] = fma2(mtwo, mul2(sy_[2], sy_[2]), one);
-        F2 u = bc(0.f), v = bc(0.f), d00 = bc(0.f), d01 = bc(0.f), d10 = bc(0.f);
+        // the sums with a negative sign are kept as their opposites (the same bits)
+        F2 un = bc(0.f), v = bc(0.f), d11 = bc(0.f), d01 = bc(0.f), d10n = bc(0.f);
 #pragma unroll
         for (int k = 1; k <= 4; ++k) {
             F2 Ux = bc(0.f), Vx = bc(0.f), W = bc(0.f);
@@ -138,13 +139,16 @@ __device__ __forceinline__ V2p vel2d_pair(const VelParams &vp, const StageCoef &
                 W = fma2(scp->All[stage][kl], sy_[l], W);
             }
             const float kp = (float)k * kPi;
-            u = fma2(neg2(s[k]), Ux, u);
-            v = fma2(mul2(bc(kp), c[k]), Vx, v);
-            d00 = fma2(mul2(bc(-kp), c[k]), Ux, d00);
+            const F2 kc = mul2(bc(kp), c[k]);
+            un = fma2(s[k], Ux, un);
+            v = fma2(kc, Vx, v);
+            d11 = fma2(kc, Ux, d11);
             d01 = fma2(s[k], W, d01);
-            d10 = fma2(mul2(bc(-kp * kp), s[k]), Vx, d10);
+            d10n = fma2(mul2(bc(kp * kp), s[k]), Vx, d10n);
         }
-        r.u = SUM ? fma2(u, bc(1.f), u0) : u; r.v = SUM ? fma2(v, bc(1.f), v0) : v; r.d00 = d00; r.d01 = d01; r.d10 = d10; r.d11 = neg2(d00);
+        r.u = SUM ? fma2(un, bc(-1.f), u0) : neg2(un);
+        r.v = SUM ? fma2(v, bc(1.f), v0) : v;
+        r.d00 = neg2(d11); r.d01 = d01; r.d10 = neg2(d10n); r.d11 = d11;
     }
     return r;
 }

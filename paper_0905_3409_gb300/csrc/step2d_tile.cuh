@@ -38,7 +38,7 @@ template <int TY, int HYV = HY, int W = TW> struct Geo {
 template <int TY, int WC> struct Smem {
     float psy[WC ? TY : 1][TX + 3];   // psi_y+ of columns x0-2 .. x0+TX
     StageCoefPair scp;
-    float fsum[12][TY];               // FOURIER2D stage 1: row sums of the tile's rows
+    __align__(8) float fsum[12][TY];  // FOURIER2D stage 1: row sums of the tile's rows
     uint64_t bar;
 };
 
@@ -88,27 +88,40 @@ __device__ __forceinline__ void fourier_row(const StageCoef &sc, float y, int k,
     }
 }
 
-// v, Dv at the two nodes (rows r, r1 of the tile) of a thread's column.
+// v, Dv at the two nodes (rows r, r1 of the tile) of a thread's column; row(q) gives row sum q
+// of both.
+template <class Row>
+__device__ __forceinline__ V2p fourier_stage1(const FCol &f, Row row)
+{
+    F2 un = bc(0.f), v = bc(0.f), d11 = bc(0.f), d01 = bc(0.f), d10n = bc(0.f);
+#pragma unroll
+    for (int k = 1; k <= 4; ++k) {
+        const F2 Ux = row(k - 1), Vx = row(4 + k - 1), W = row(8 + k - 1);
+        const float kp = (float)k * kPi;
+        const F2 sk = bc(f.s[k]), kc = mul2(bc(kp), bc(f.c[k]));
+        un = fma2(sk, Ux, un);
+        v = fma2(kc, Vx, v);
+        d11 = fma2(kc, Ux, d11);
+        d01 = fma2(sk, W, d01);
+        d10n = fma2(mul2(bc(kp * kp), sk), Vx, d10n);
+    }
+    V2p rr;
+    rr.u = neg2(un); rr.v = v; rr.d00 = neg2(d11); rr.d01 = d01; rr.d10 = neg2(d10n); rr.d11 = d11;
+    return rr;
+}
+
 template <int TY>
 __device__ __forceinline__ V2p fourier_stage1_pair(const FCol &f, const float (*fsum)[TY], int r, int r1)
 {
-    F2 u = bc(0.f), v = bc(0.f), d00 = bc(0.f), d01 = bc(0.f), d10 = bc(0.f);
-#pragma unroll
-    for (int k = 1; k <= 4; ++k) {
-        const F2 Ux = make_float2(fsum[k - 1][r], fsum[k - 1][r1]);
-        const F2 Vx = make_float2(fsum[4 + k - 1][r], fsum[4 + k - 1][r1]);
-        const F2 W = make_float2(fsum[8 + k - 1][r], fsum[8 + k - 1][r1]);
-        const float kp = (float)k * kPi;
-        const F2 sk = bc(f.s[k]), ck = bc(f.c[k]);
-        u = fma2(neg2(sk), Ux, u);
-        v = fma2(mul2(bc(kp), ck), Vx, v);
-        d00 = fma2(mul2(bc(-kp), ck), Ux, d00);
-        d01 = fma2(sk, W, d01);
-        d10 = fma2(mul2(bc(-kp * kp), sk), Vx, d10);
-    }
-    V2p rr;
-    rr.u = u; rr.v = v; rr.d00 = d00; rr.d01 = d01; rr.d10 = d10; rr.d11 = neg2(d00);
-    return rr;
+    return fourier_stage1(f, [&](int q) { return make_float2(fsum[q][r], fsum[q][r1]); });
+}
+
+// The same for rows r, r + 1 (r even): one 8-byte load per sum.
+template <int TY>
+__device__ __forceinline__ V2p fourier_stage1_next(const FCol &f, const float (*fsum)[TY], int r)
+{
+    static_assert(TY % 2 == 0, "row pairs are 8-byte aligned");
+    return fourier_stage1(f, [&](int q) { return *reinterpret_cast<const float2 *>(&fsum[q][r]); });
 }
 
 // phi_xy at corner column q (q = k + o, o in {0,1}) from the psi_y row window
@@ -445,7 +458,7 @@ __device__ __forceinline__ bool tile_step2d(const float *__restrict__ in, float 
             const Sep2 ry = (VK == VK_VORTEX2D) ? sep_factors2(y) : Sep2{bc(0.f), bc(0.f), bc(0.f)};
             F2 phi, px, py;
             if (VK == VK_FOURIER2D && TR != TR_GIVEN) {
-                const V2p a1 = fourier_stage1_pair<TY>(fcol, sm.fsum, r, r + 1);
+                const V2p a1 = fourier_stage1_next<TY>(fcol, sm.fsum, r);
                 node2d_pair<TY, TR, VK, CR, HYV, COH, W, OV>(in, g, tile, gx0, y0, vp, sc, scp, dt, i, j0, i,
                                                    j1, x, y, cx, ry, phi, px, py, &a1);
             } else {
