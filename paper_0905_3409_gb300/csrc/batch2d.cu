@@ -10,7 +10,7 @@
 // the SM count) the blocks are persistent and re-use their shared memory and barrier
 // (one mbarrier phase per tile).
 #include "batch_internal.h"
-#include "step2d_tile.cuh"
+#include "step2d_walk.cuh"
 
 namespace gals {
 
@@ -18,15 +18,25 @@ namespace {
 
 using namespace t2;
 
+// Whether the steps that write no phi_xy walk their tiles (as on one grid: the Fourier field's
+// tables leave no registers for the carried rows).
+template <int VK, int WC> constexpr bool walked() { return !WC && VK != VK_FOURIER2D; }
+
+template <int TY, int VK, int WC> struct BatchSmemOf { using T = Smem<TY, WC>; };
+template <int TY> struct BatchSmemOf<TY, VK_VORTEX2D, 0> { using T = WalkSmem<TY>; };
+template <int TY> struct BatchSmemOf<TY, VK_ROTATION, 0> { using T = WalkSmem<TY>; };
+
+// Blocks per SM: the steps between the first and the last of a run (no phi_xy plane, no
+// exchange of psi_y) fit five.
 template <int TY, int VK, int CR, int WC>
-__global__ void __launch_bounds__(TX, 4)
+__global__ void __launch_bounds__(TX, WC ? 4 : 5)
 k_batch2d(const float *__restrict__ in_base, float *__restrict__ out_base,
           const BatchProb *__restrict__ probs, const VelParams *__restrict__ vps,
           const StageCoef *__restrict__ coef, const CUtensorMap *__restrict__ maps,
           const BatchItem *__restrict__ items, int nitems, int *__restrict__ err)
 {
     extern __shared__ __align__(128) float tile[];
-    __shared__ __align__(16) Smem<TY, WC> sm;
+    __shared__ __align__(16) typename BatchSmemOf<TY, VK, WC>::T sm;
     if (threadIdx.x == 0) mbar_init(&sm.bar, 1);
     __syncthreads();
     uint32_t parity = 0;
@@ -34,9 +44,15 @@ k_batch2d(const float *__restrict__ in_base, float *__restrict__ out_base,
         const BatchItem w = items[it];
         const BatchProb &P = probs[w.prob];
         const Geom g = P.g;
-        const bool ok = tile_step2d<TY, TR_RK3, VK, CR, WC>(
-            in_base + P.off, out_base + P.off, g, vps[w.prob], coef + w.prob, P.dt,
-            maps + w.prob, err, w.x0, w.y0, tile, sm, parity);
+        bool ok;
+        if constexpr (walked<VK, WC>())
+            ok = tile_walk2d<TY, TR_RK3, VK, CR, HY, TW>(in_base + P.off, out_base + P.off, g, vps[w.prob],
+                                                         coef + w.prob, P.dt, maps + w.prob, err, w.x0, w.y0, g.n1,
+                                                         tile, sm, parity);
+        else
+            ok = tile_step2d<TY, TR_RK3, VK, CR, WC>(in_base + P.off, out_base + P.off, g, vps[w.prob],
+                                                     coef + w.prob, P.dt, maps + w.prob, err, w.x0, w.y0, tile, sm,
+                                                     parity);
         if (!ok) return;  // block-uniform
         parity ^= 1u;
         __syncthreads();  // tile and psi_y buffers are free before the next copy
@@ -157,7 +173,7 @@ cudaError_t launch_t(const BatchLaunch &a, cudaStream_t s)
         attr_set = true;
     }
     const int grid = a.grid > 0 ? a.grid : a.nitems;
-    kern<<<grid, TX, Geo<TY>::bytes(NP), s>>>(a.in, a.out, a.probs, a.vps, a.coef, a.maps,
+    kern<<<grid, TX, Geo<TY>::bytes(NP), s>>>(a.in, a.out, a.probs, a.vps, a.coef, a.maps[NP - 3],
                                               a.items, a.nitems, a.err);
     return cudaGetLastError();
 }
@@ -208,7 +224,9 @@ cudaError_t launch_run_kind(const BatchRunLaunch &a, cudaStream_t s)
 template <int TY, int VK>
 cudaError_t launch_layout(const BatchLaunch &a, cudaStream_t s)
 {
-    return a.compact ? launch_t<TY, VK, CROSS_RECON, 0>(a, s) : launch_t<TY, VK, CROSS_PLANE, 1>(a, s);
+    if (a.cross_in == CROSS_PLANE)
+        return a.write_cross ? launch_t<TY, VK, CROSS_PLANE, 1>(a, s) : launch_t<TY, VK, CROSS_PLANE, 0>(a, s);
+    return a.write_cross ? launch_t<TY, VK, CROSS_RECON, 1>(a, s) : launch_t<TY, VK, CROSS_RECON, 0>(a, s);
 }
 
 template <int TY>
@@ -238,16 +256,13 @@ void batch_tile_box(int variant, int np, uint32_t box[3])
     box[2] = (uint32_t)np;
 }
 
-int batch_max_blocks_per_sm(int variant, int kind, int compact)
+int batch_max_blocks_per_sm(int variant, int kind)
 {
     // occupancy of the kernel actually launched (registers and shared memory)
     int nb = 0;
-    const int np = compact ? 3 : 4;
-    const int bytes = variant == 0 ? Geo<8>::bytes(np) : Geo<16>::bytes(np);
+    const int bytes = variant == 0 ? Geo<8>::bytes(3) : Geo<16>::bytes(3);
     cudaError_t e = cudaSuccess;
-#define OCC(TY, VK)                                                                             \
-    e = compact ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch2d<TY, VK, CROSS_RECON, 0>, TX, bytes) \
-                : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch2d<TY, VK, CROSS_PLANE, 1>, TX, bytes)
+#define OCC(TY, VK) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_batch2d<TY, VK, CROSS_RECON, 0>, TX, bytes)
     if (variant == 0) {
         if (kind == VK_FOURIER2D) OCC(8, VK_FOURIER2D); else if (kind == VK_VORTEX2D) OCC(8, VK_VORTEX2D); else OCC(8, VK_ROTATION);
     } else {

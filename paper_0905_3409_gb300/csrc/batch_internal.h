@@ -23,13 +23,14 @@ struct BatchLaunch {
     const BatchProb *probs;
     const VelParams *vps;    // per-problem velocity parameters
     const StageCoef *coef;   // this step's coefficients, one per problem
-    const CUtensorMap *maps; // per-problem TMA maps of `in`
+    const CUtensorMap *maps[2]; // per-problem TMA maps of `in`: phi and psi; all planes (FULL)
     const BatchItem *items;
     int nitems;
     int grid;                // blocks (0: one per item)
     int variant;             // 0: 128 x 8 tiles, 1: 128 x 16 tiles
     int kind;                // velocity kind shared by all problems
-    int compact;             // COMPACT layout (mixed derivatives rebuilt on the fly)
+    int cross_in;            // CROSS_PLANE: read the stored phi_xy; CROSS_RECON: rebuild it
+    int write_cross;         // write the new phi_xy plane
     int *err;
 };
 
@@ -54,7 +55,8 @@ bool batch_kind_supported(int kind);
 cudaError_t launch_batch2d_run(const BatchRunLaunch &a, cudaStream_t s);
 int batch_tile_rows(int variant);
 void batch_tile_box(int variant, int np, uint32_t box[3]);
-int batch_max_blocks_per_sm(int variant, int kind, int compact);
+// Resident blocks per SM of the kernel that steps between the first and the last of a run.
+int batch_max_blocks_per_sm(int variant, int kind);
 cudaError_t launch_batch2d(const BatchLaunch &a, cudaStream_t s);
 cudaError_t launch_batch_coef(StageCoef *table, const VelParams *vps, const double *t_dev,
                               const BatchProb *probs, int nprob, int nsteps, cudaStream_t s);
