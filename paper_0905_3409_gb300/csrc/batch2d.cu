@@ -142,15 +142,19 @@ k_batch2d_run(float *__restrict__ buf0, float *__restrict__ buf1, const BatchPro
     }
 }
 
-__global__ void k_batch_coef(StageCoef *table, const VelParams *__restrict__ vps,
-                             const double *__restrict__ t_dev, const BatchProb *__restrict__ probs,
-                             int nprob, int nsteps)
+constexpr int kCoefWarps = 4;
+
+// One warp per problem and step.
+__global__ void __launch_bounds__(32 * kCoefWarps)
+k_batch_coef(StageCoef *table, const VelParams *__restrict__ vps, const double *__restrict__ t_dev,
+             const BatchProb *__restrict__ probs, int nprob, int nsteps)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double term[kCoefWarps][3 * kMaxModes];
+    const int w = threadIdx.x >> 5, e = blockIdx.x * kCoefWarps + w;
     if (e >= nprob * nsteps) return;
     const int p = e % nprob, s = e / nprob;
     const double dt = probs[p].dt_d;
-    stage_coef_one(vps[p], t_dev[p] + (double)s * dt, dt, table[e]);
+    stage_coef_warp(vps[p], t_dev[p] + (double)s * dt, dt, table[e], term[w]);
 }
 
 __global__ void k_batch_advance(double *t_dev, const BatchProb *__restrict__ probs, int nprob,
@@ -287,7 +291,7 @@ cudaError_t launch_batch_coef(StageCoef *table, const VelParams *vps, const doub
                               const BatchProb *probs, int nprob, int nsteps, cudaStream_t s)
 {
     const int n = nprob * nsteps;
-    k_batch_coef<<<(n + 127) / 128, 128, 0, s>>>(table, vps, t_dev, probs, nprob, nsteps);
+    k_batch_coef<<<(n + kCoefWarps - 1) / kCoefWarps, 32 * kCoefWarps, 0, s>>>(table, vps, t_dev, probs, nprob, nsteps);
     return cudaGetLastError();
 }
 

@@ -25,14 +25,17 @@ __global__ void k_set_time(double *t, double value)
 }  // namespace
 
 namespace {
-__global__ void k_coef_table(StageCoef *table, VelParams vp, const double *t_dev, double dt,
-                             int nsteps)
+constexpr int kCoefWarps = 8;
+
+// One warp per step of a run.
+__global__ void __launch_bounds__(32 * kCoefWarps)
+k_coef_table(StageCoef *table, const __grid_constant__ VelParams vp, const double *t_dev, double dt, int nsteps)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    __shared__ double term[kCoefWarps][3 * kMaxModes];
+    const int w = threadIdx.x >> 5, k = blockIdx.x * kCoefWarps + w;
     if (k >= nsteps) return;
-    const double t = t_dev[0] + (double)k * dt;
-    stage_coef_one(vp, t, dt, table[k]);
-    if (vp.kind == VK_WAVES2D) table[k].wamp = vp.wamp + (size_t)k * 3 * vp.nwaves;
+    stage_coef_warp(vp, t_dev[0] + (double)k * dt, dt, table[k], term[w]);
+    if (vp.kind == VK_WAVES2D && (threadIdx.x & 31) == 3) table[k].wamp = vp.wamp + (size_t)k * 3 * vp.nwaves;
 }
 
 // WAVES2D amplitudes of the call's steps: wamp[(k 3 + s) M + m] = a_m cos(2 pi (n_m t_s + chi_m'))
@@ -61,7 +64,7 @@ cudaError_t launch_coef_table(StageCoef *table, const VelParams &vp, const doubl
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    k_coef_table<<<(nsteps + 63) / 64, 64, 0, s>>>(table, vp, t_dev, dt, nsteps);
+    k_coef_table<<<(nsteps + kCoefWarps - 1) / kCoefWarps, 32 * kCoefWarps, 0, s>>>(table, vp, t_dev, dt, nsteps);
     return cudaGetLastError();
 }
 
