@@ -5,6 +5,7 @@
 // and phases, RK4 flow-map targets), runs the forward and backward kernels and an Adam
 // update with a cosine learning-rate schedule; the output scales (one per output) are the
 // standard deviations of a calibration batch, so the network works on O(1) targets.
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdarg>
@@ -24,10 +25,17 @@ struct gals_surrogate {
     InferParams ip{};
     float *scale_dev = nullptr, *one = nullptr;
     double *loss_dev = nullptr;
-    // training scratch (capacity `cap` samples)
-    int cap = 0;
-    float *Xn = nullptr, *T = nullptr, *Z[NLAYER] = {}, *A[NLAYER] = {}, *G0 = nullptr, *G1 = nullptr;
-    float *split = nullptr;
+    // inputs and targets / outputs (capacity `cap` rows)
+    int64_t cap = 0;
+    float *Xn = nullptr, *T = nullptr;
+    // training scratch of the general path (capacity `gen_cap` samples)
+    int gen_cap = 0;
+    float *Z[NLAYER] = {}, *A[NLAYER] = {}, *G0 = nullptr, *G1 = nullptr, *split = nullptr;
+    // and of the fused one (capacity `tile_cap` chunks): pre-activations, partial gradients,
+    // packed weights
+    int tile_cap = 0;
+    float *Zs = nullptr, *part = nullptr;
+    uint16_t *wt = nullptr;
     // bound field
     bool bound = false;
     VelParams vp{};
@@ -86,17 +94,44 @@ uint64_t splitmix64_host(uint64_t &state)
     return z ^ (z >> 31);
 }
 
-cudaError_t ensure_scratch(gals_surrogate *s, int n)
+// Room for n rows of inputs and of targets or outputs.
+cudaError_t ensure_io(gals_surrogate *s, int64_t n)
 {
     if (n <= s->cap) return cudaSuccess;
     cudaStreamSynchronize(s->stream);
-    cudaFree(s->Xn); cudaFree(s->T); cudaFree(s->G0); cudaFree(s->G1); cudaFree(s->split);
-    for (int l = 0; l < NLAYER; ++l) { cudaFree(s->Z[l]); cudaFree(s->A[l]); s->Z[l] = s->A[l] = nullptr; }
-    s->Xn = s->T = s->G0 = s->G1 = s->split = nullptr;
+    cudaFree(s->Xn); cudaFree(s->T);
+    s->Xn = s->T = nullptr;
     s->cap = 0;
     cudaError_t e;
-    if ((e = cudaMalloc(&s->Xn, sizeof(float) * 3 * (size_t)n)) != cudaSuccess) return e;
+    if ((e = cudaMalloc(&s->Xn, sizeof(float) * IN * (size_t)n)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&s->T, sizeof(float) * OUT * (size_t)n)) != cudaSuccess) return e;
+    s->cap = n;
+    return cudaSuccess;
+}
+
+// Scratch of forward and backward passes over n samples.
+cudaError_t ensure_train(gals_surrogate *s, int n)
+{
+    cudaError_t e;
+    if (n <= kFusedBatch) {
+        const int tiles = train_splits(n);
+        if (tiles <= s->tile_cap) return cudaSuccess;
+        cudaStreamSynchronize(s->stream);
+        cudaFree(s->Zs); cudaFree(s->part);
+        s->Zs = s->part = nullptr;
+        s->tile_cap = 0;
+        if ((e = cudaMalloc(&s->Zs, sizeof(float) * 4 * 128 * HID * (size_t)tiles)) != cudaSuccess) return e;
+        if ((e = cudaMalloc(&s->part, sizeof(float) * kPartStride * (size_t)tiles)) != cudaSuccess) return e;
+        if (!s->wt && (e = cudaMalloc(&s->wt, sizeof(uint16_t) * train_weights_elems())) != cudaSuccess) return e;
+        s->tile_cap = tiles;
+        return cudaSuccess;
+    }
+    if (n <= s->gen_cap) return cudaSuccess;
+    cudaStreamSynchronize(s->stream);
+    cudaFree(s->G0); cudaFree(s->G1); cudaFree(s->split);
+    for (int l = 0; l < NLAYER; ++l) { cudaFree(s->Z[l]); cudaFree(s->A[l]); s->Z[l] = s->A[l] = nullptr; }
+    s->G0 = s->G1 = s->split = nullptr;
+    s->gen_cap = 0;
     if ((e = cudaMalloc(&s->G0, sizeof(float) * HID * (size_t)n)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&s->G1, sizeof(float) * HID * (size_t)n)) != cudaSuccess) return e;
     if ((e = cudaMalloc(&s->split, sizeof(float) * kMaxSplit * HID * HID)) != cudaSuccess) return e;
@@ -104,8 +139,24 @@ cudaError_t ensure_scratch(gals_surrogate *s, int n)
         if ((e = cudaMalloc(&s->Z[l], sizeof(float) * lout(l) * (size_t)n)) != cudaSuccess) return e;
         if (l > 0 && (e = cudaMalloc(&s->A[l], sizeof(float) * HID * (size_t)n)) != cudaSuccess) return e;
     }
-    s->cap = n;
+    s->gen_cap = n;
     return cudaSuccess;
+}
+
+// Gradient and loss of the n samples X, T by the path that serves their number.
+cudaError_t loss_gradient(gals_surrogate *s, const float *X, const float *T, int n)
+{
+    cudaError_t e;
+    if (n <= kFusedBatch) {
+        if ((e = pack_train(s->params, s->wt, s->stream)) != cudaSuccess ||
+            (e = launch_train_tiles(s->params, s->wt, X, T, n, s->Zs, s->part, s->loss_dev, s->err_dev, s->stream)) !=
+                cudaSuccess)
+            return e;
+        return launch_train_grad(s->part, n, s->grad, s->stream);
+    }
+    if ((e = forward_train(s->params, X, n, s->Z, s->A, s->err_dev, s->stream)) != cudaSuccess) return e;
+    return backward_train(s->params, X, T, n, s->Z, s->A, s->G0, s->G1, s->grad, s->loss_dev, s->one, s->split,
+                          s->err_dev, s->stream);
 }
 
 gals_status check_field(gals_surrogate *s, const gals_velocity *vel, VelParams &vp)
@@ -243,6 +294,7 @@ gals_status gals_surrogate_destroy(gals_surrogate *s)
     cudaFree(s->ip.w); cudaFree(s->scale_dev); cudaFree(s->one);
     cudaFree(s->loss_dev); cudaFree(s->counters); cudaFree(s->err_dev);
     cudaFree(s->Xn); cudaFree(s->T); cudaFree(s->G0); cudaFree(s->G1); cudaFree(s->split);
+    cudaFree(s->Zs); cudaFree(s->part); cudaFree(s->wt);
     for (int l = 0; l < NLAYER; ++l) { cudaFree(s->Z[l]); cudaFree(s->A[l]); }
     if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
     delete s;
@@ -265,12 +317,17 @@ gals_status gals_surrogate_train(gals_surrogate *s, const gals_velocity *vel, do
     if (st != GALS_OK) return st;
     const auto t0 = std::chrono::steady_clock::now();
     cudaError_t e;
-    if ((e = ensure_scratch(s, o->batch)) != cudaSuccess) return scuda(s, e, "training scratch");
-    // output scales: standard deviations of a calibration batch (scale 1 first)
     const int n = o->batch;
+    const bool fused = n <= kFusedBatch;
+    // samples of several steps per launch (they do not depend on the weights): about a
+    // quarter of a million threads
+    const int group = std::min(o->steps, std::max(1, (1 << 18) / n));
+    if ((e = ensure_io(s, (int64_t)n * group)) != cudaSuccess || (e = ensure_train(s, n)) != cudaSuccess)
+        return scuda(s, e, "training scratch");
+    // output scales: standard deviations of a calibration batch (scale 1 first)
     std::vector<float> ones(OUT, 1.f), Th((size_t)n * OUT);
     if ((e = cudaMemcpyAsync(s->scale_dev, ones.data(), sizeof(float) * OUT, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess ||
-        (e = launch_samples(vp, s->Xn, s->T, n, (float)dt, (float)h, o->substeps, o->seed ^ 0xC0FFEEull, 0,
+        (e = launch_samples(vp, s->Xn, s->T, n, (float)dt, (float)h, o->substeps, o->seed ^ 0xC0FFEEull, 0, 1,
                             s->scale_dev, s->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(Th.data(), s->T, sizeof(float) * Th.size(), cudaMemcpyDeviceToHost, s->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s->stream)) != cudaSuccess)
@@ -286,20 +343,31 @@ gals_status gals_surrogate_train(gals_surrogate *s, const gals_velocity *vel, do
     }
     if ((e = cudaMemcpyAsync(s->scale_dev, scale, sizeof(scale), cudaMemcpyHostToDevice, s->stream)) != cudaSuccess)
         return scuda(s, e, "scales");
+    if (fused && (e = pack_train(s->params, s->wt, s->stream)) != cudaSuccess) return scuda(s, e, "pack");
     double first = -1.0, last = 0.0;
     for (int it = 0; it < o->steps; ++it) {
-        if ((e = launch_samples(vp, s->Xn, s->T, n, (float)dt, (float)h, o->substeps, o->seed, (uint64_t)it + 1,
-                                s->scale_dev, s->stream)) != cudaSuccess ||
-            (e = forward_train(s->params, s->Xn, n, s->Z, s->A, s->err_dev, s->stream)) != cudaSuccess ||
-            (e = backward_train(s->params, s->Xn, s->T, n, s->Z, s->A, s->G0, s->G1, s->grad, s->loss_dev,
-                                s->one, s->split, s->err_dev, s->stream)) != cudaSuccess)
-            return scuda(s, e, "training step");
+        const int at = it % group;
+        if (at == 0 && (e = launch_samples(vp, s->Xn, s->T, n, (float)dt, (float)h, o->substeps, o->seed,
+                                           (uint64_t)it + 1, std::min(group, o->steps - it), s->scale_dev,
+                                           s->stream)) != cudaSuccess)
+            return scuda(s, e, "training samples");
+        const float *X = s->Xn + (size_t)at * IN * n, *T = s->T + (size_t)at * OUT * n;
         const double frac = o->steps > 1 ? (double)it / (o->steps - 1) : 0.0;
         const double lr = o->lr_min + 0.5 * (o->lr - o->lr_min) * (1.0 + std::cos(M_PI * frac));
-        if ((e = adam_step(s->params, s->grad, s->m, s->v, (float)lr, 0.9f, 0.999f, 1e-8f, ++s->adam_step,
-                           s->stream)) != cudaSuccess)
-            return scuda(s, e, "adam");
-        if (it == 0 || it == o->steps - 1) {
+        const bool report_loss = it == 0 || it == o->steps - 1;
+        if (fused) {
+            if ((e = launch_train_tiles(s->params, s->wt, X, T, n, s->Zs, s->part, report_loss ? s->loss_dev : nullptr,
+                                        s->err_dev, s->stream)) != cudaSuccess ||
+                (e = launch_train_adam(s->part, n, s->params, s->m, s->v, s->wt, (float)lr, 0.9f, 0.999f, 1e-8f,
+                                       ++s->adam_step, s->stream)) != cudaSuccess)
+                return scuda(s, e, "training step");
+        } else {
+            if ((e = loss_gradient(s, X, T, n)) != cudaSuccess) return scuda(s, e, "training step");
+            if ((e = adam_step(s->params, s->grad, s->m, s->v, (float)lr, 0.9f, 0.999f, 1e-8f, ++s->adam_step,
+                               s->stream)) != cudaSuccess)
+                return scuda(s, e, "adam");
+        }
+        if (report_loss) {
             double l = 0.0;
             if ((e = cudaMemcpyAsync(&l, s->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, s->stream)) != cudaSuccess ||
                 (e = cudaStreamSynchronize(s->stream)) != cudaSuccess)
@@ -398,7 +466,7 @@ gals_status gals_surrogate_forward(gals_surrogate *s, const float *inputs, int n
 {
     if (!s || !inputs || !outputs || n < 1 || n > 65536) return sfail(s, GALS_ERR_ARG, "bad arguments");
     cudaError_t e;
-    if ((e = ensure_scratch(s, n)) != cudaSuccess) return scuda(s, e, "scratch");
+    if ((e = ensure_io(s, n)) != cudaSuccess) return scuda(s, e, "scratch");
     if ((e = cudaMemcpyAsync(s->Xn, inputs, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess ||
         (e = infer_points(s->ip, s->Xn, s->T, n, s->err_dev, s->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(outputs, s->T, sizeof(float) * OUT * n, cudaMemcpyDeviceToHost, s->stream)) != cudaSuccess ||
@@ -420,13 +488,11 @@ gals_status gals_surrogate_gradient(gals_surrogate *s, const float *inputs, cons
 {
     if (!s || !inputs || !targets || !grad || n < 1 || n > 65536) return sfail(s, GALS_ERR_ARG, "bad arguments");
     cudaError_t e;
-    if ((e = ensure_scratch(s, n)) != cudaSuccess) return scuda(s, e, "scratch");
+    if ((e = ensure_io(s, n)) != cudaSuccess || (e = ensure_train(s, n)) != cudaSuccess) return scuda(s, e, "scratch");
     double l = 0.0;
     if ((e = cudaMemcpyAsync(s->Xn, inputs, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(s->T, targets, sizeof(float) * OUT * n, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess ||
-        (e = forward_train(s->params, s->Xn, n, s->Z, s->A, s->err_dev, s->stream)) != cudaSuccess ||
-        (e = backward_train(s->params, s->Xn, s->T, n, s->Z, s->A, s->G0, s->G1, s->grad, s->loss_dev, s->one,
-                            s->split, s->err_dev, s->stream)) != cudaSuccess ||
+        (e = loss_gradient(s, s->Xn, s->T, n)) != cudaSuccess ||
         (e = cudaMemcpyAsync(grad, s->grad, sizeof(float) * NPARAM, cudaMemcpyDeviceToHost, s->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(&l, s->loss_dev, sizeof(double), cudaMemcpyDeviceToHost, s->stream)) != cudaSuccess ||
         (e = cudaStreamSynchronize(s->stream)) != cudaSuccess)
@@ -446,7 +512,7 @@ gals_status gals_surrogate_targets(gals_surrogate *s, const gals_velocity *vel, 
     gals_status st = check_field(s, vel, vp);
     if (st != GALS_OK) return st;
     cudaError_t e;
-    if ((e = ensure_scratch(s, n)) != cudaSuccess) return scuda(s, e, "scratch");
+    if ((e = ensure_io(s, n)) != cudaSuccess) return scuda(s, e, "scratch");
     if ((e = cudaMemcpyAsync(s->Xn, points, sizeof(float) * 3 * n, cudaMemcpyHostToDevice, s->stream)) != cudaSuccess ||
         (e = launch_targets(vp, s->Xn, s->T, n, (float)dt, (float)h, substeps, s->stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(targets, s->T, sizeof(float) * OUT * n, cudaMemcpyDeviceToHost, s->stream)) != cudaSuccess ||

@@ -45,6 +45,17 @@ __device__ __forceinline__ float silu_prime(float z)
     return fmaf(z * s, 1.f - s, s);
 }
 
+// One Adam update of parameter i with gradient gi (c1, c2: the bias corrections).
+__device__ __forceinline__ void adam_update(float *p, float gi, float *m, float *v, int64_t i, float lr, float b1,
+                                            float b2, float eps, float c1, float c2)
+{
+    const float mi = b1 * m[i] + (1.f - b1) * gi;
+    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
 __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__float2bfloat16(v)); }
 
 }  // namespace mlp

@@ -36,14 +36,11 @@ struct Check {
     int *err;                               // device error word (bounded waits)
 };
 
-__device__ void flowmap_rk4(const VelParams &vp, float x, float y, float t, float dt, int m,
-                            float d[2], float J[4]);
-
 cudaError_t launch_targets(const VelParams &vp, const float *X, float *T, int n, float dt, float h,
                            int substeps, cudaStream_t s);
 cudaError_t launch_samples(const VelParams &vp, float *Xn, float *T, int n, float dt, float h,
-                           int substeps, uint64_t seed, uint64_t step, const float *scale,
-                           cudaStream_t s);
+                           int substeps, uint64_t seed, uint64_t step, int nsteps, const float *scale,
+                           cudaStream_t s);  // samples of nsteps steps, one after the other
 // Training products on the tensor cores; a product that does not complete in time sets *err.
 cudaError_t forward_train(const float *params, const float *X, int n, float *const *Z,
                           float *const *A, int *err, cudaStream_t s);
@@ -52,6 +49,22 @@ constexpr int kMaxSplit = 128;
 cudaError_t backward_train(const float *params, const float *X, const float *T, int n,
                            float *const *Z, float *const *A, float *G0, float *G1, float *grad,
                            double *loss, const float *one, float *split, int *err, cudaStream_t s);
+// split-K chunks of the weight gradients: at least 128 samples each, at most kMaxSplit
+inline int train_splits(int n) { return (n + 127) / 128 < kMaxSplit ? (n + 127) / 128 : kMaxSplit; }
+// Forward and backward pass of a step in one launch (mlp_train_tile.cu), for batches whose
+// chunks fit a block's 128 rows.  wt: packed BF16 weights (pack_train, kept up to date by
+// launch_train_adam); Zs: train_splits(n) * 4 * 128 * 128 floats; part: train_splits(n) *
+// kPartStride floats of partial gradients, which launch_train_grad sums and
+// launch_train_adam sums and applies; loss may be null.
+constexpr int kFusedBatch = 128 * kMaxSplit;
+constexpr int kPartStride = (int)((NPARAM + 3) / 4 * 4);
+int64_t train_weights_elems();
+cudaError_t pack_train(const float *params, uint16_t *wt, cudaStream_t s);
+cudaError_t launch_train_tiles(const float *params, const uint16_t *wt, const float *X, const float *T, int n,
+                               float *Zs, float *part, double *loss, int *err, cudaStream_t s);
+cudaError_t launch_train_grad(const float *part, int n, float *grad, cudaStream_t s);
+cudaError_t launch_train_adam(const float *part, int n, float *params, float *m, float *v, uint16_t *wt, float lr,
+                              float b1, float b2, float eps, int step, cudaStream_t s);
 cudaError_t adam_step(float *params, const float *grad, float *m, float *v, float lr, float b1,
                       float b2, float eps, int step, cudaStream_t s);
 // FP32 master parameters -> inference layout
