@@ -150,15 +150,33 @@ gals_status make_velparams(gals_grid *g, const gals_velocity *v, VelParams &vp)
     return GALS_OK;
 }
 
+// Whether the steps of a FULL 3D run rebuild the mixed derivatives (step_launch): while few
+// feet leave the staged tile, one cell around it.  The deformation field's bound is reached
+// by one component at a few nodes (half of it stands for the field), a rotation's by an
+// edge of the box.  Measured, us per step, rebuilt against reconstructed: 256^3 deformation
+// at CFL 1 / 2 / 4 344 against 351, 345 against 352, 386 against 379; rotation at CFL 1 / 2
+// 306 against 311, 450 against 398; 101^3 deformation at CFL 2 33.2 against 37.4.
+// The Heun form evaluates a velocity more after the interpolant and has no registers to
+// spare there: above a few million nodes, where the saved launch does not count, it keeps the
+// pass (200 x 190 x 180 deformation 167 us against 161, rotation 142 against 134; 101^3 33.7
+// against 36.1).
+bool rebuild3d(int kind, int trace, int64_t nodes, double reach)
+{
+    return (kind == GALS_VEL_DEFORM3D ? 0.5 * reach : reach) <= 1.05 &&
+           (trace != GALS_TRACE_HEUN_PSI || nodes <= 2000000);
+}
+
 // Kernel launch descriptor of step s of a run of nsteps, from buffer cur to buffer cur ^ 1.
 // Between the steps of a run nobody reads the mixed derivatives of approach A but the next
 // step, so only the run's first step reads their stored planes and only its last one
 // writes them; the steps between rebuild them from the gradients around each cell (the
 // COMPACT layout's way, the same stencils and bits).  In 2D that moves 24 instead of 32
 // bytes per node and leaves out the exchange of psi_y+ at the end of a tile: 4096^2 vortex
-// 119.4 us per step against 128.5 (107.8 with the walked tiles of step2d_walk.cuh).
+// 119.4 us per step against 128.5 (107.8 with the walked tiles of step2d_walk.cuh).  In 3D
+// rebuilding costs about what the reconstruction pass does, and feet that leave the staged
+// tile cost more: `rebuild` says whether it is the faster way (rebuild3d).
 StepLaunch step_launch(gals_grid *g, const VelParams &vp, int trace, double dt, int s, int nsteps, int cur,
-                       bool first_explicit)
+                       bool first_explicit, bool rebuild = true)
 {
     StepLaunch a{};
     a.in = g->buf[cur];
@@ -178,8 +196,8 @@ StepLaunch step_launch(gals_grid *g, const VelParams &vp, int trace, double dt, 
         a.cross_in = CROSS_CELL;  // approach B: mixed derivatives per cell, none stored
         a.write_cross = 0;
     } else if (g->layout == GALS_LAYOUT_FULL) {
-        a.cross_in = (s == 0 || g->dim == 3) ? CROSS_PLANE : CROSS_RECON;
-        a.write_cross = s == nsteps - 1 || g->dim == 3;
+        a.cross_in = s == 0 || !rebuild ? CROSS_PLANE : CROSS_RECON;
+        a.write_cross = s == nsteps - 1 || !rebuild;
     } else {
         a.cross_in = (s == 0 && first_explicit) ? CROSS_PLANE : CROSS_RECON;
         a.write_cross = 0;
@@ -262,7 +280,8 @@ cudaError_t make_band_streams(gals_grid *g)
 // coefficient table and clock kernels included).
 cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt, int nsteps,
                         bool first_explicit, int64_t &launches, const mlp::InferParams *ip = nullptr,
-                        const mlp::Check *chk = nullptr, bool run = false, const StepBands *bands = nullptr)
+                        const mlp::Check *chk = nullptr, bool run = false, const StepBands *bands = nullptr,
+                        bool rebuild = true)
 {
     int cur = g->cur;
     launches = (vp.kind == VK_WAVES2D ? 2 : 1) + 1;  // coefficients (+ wave amplitudes), clock
@@ -326,7 +345,7 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
         return launch_advance_time(g->t_dev, nsteps, dt, g->stream);
     }
     for (int s = 0; s < nsteps; ++s) {
-        StepLaunch a = step_launch(g, vp, trace, dt, s, nsteps, cur, first_explicit);
+        StepLaunch a = step_launch(g, vp, trace, dt, s, nsteps, cur, first_explicit, rebuild);
         if (trace == GALS_TRACE_SURROGATE) {
             // learned trace of this step (with RK3 fallback per tile), then the Hermite stage
             ce = mlp::launch_mlp_trace(*ip, g->geom, vp, g->coef + s, g->t_dev, s, dt, g->trace_buf,
@@ -701,6 +720,8 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
     }
     const double vmax = speed_bound(v, g->dim, g->lo, g->hi);
     const double reach[2] = {dt * vmax / g->h[0], dt * vmax / g->h[1]};
+    const bool rebuild = g->dim == 2 || rebuild3d(v->kind, v->trace, (int64_t)g->n[0] * g->n[1] * g->n[2],
+                                                      std::max({reach[0], reach[1], dt * vmax / g->h[2]}));
     const bool run = use_run(g, v->trace, std::min(nsteps, kGraphSteps), reach);
     if (run && !g->run_ctl) {
         if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return cuda_fail(g, e, "sync");
@@ -744,7 +765,7 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
                 return ce;
             }
             int64_t nl = 0;
-            const cudaError_t le = issue_steps(g, vp, v->trace, dt, cs, fe_c, nl, &ip, &chk, run, &bands);
+            const cudaError_t le = issue_steps(g, vp, v->trace, dt, cs, fe_c, nl, &ip, &chk, run, &bands, rebuild);
             ce = cudaStreamEndCapture(g->stream, &graph);
             if (le != cudaSuccess) {
                 if (ce == cudaSuccess) cudaGraphDestroy(graph);

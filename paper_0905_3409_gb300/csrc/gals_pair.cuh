@@ -442,8 +442,61 @@ __device__ __forceinline__ void trace3d_pair(const V3p &a, const VelParams &vp, 
         J[e] = fma2(m6, S[e], (e % 4) == 0 ? fma2(m23, N[e], one) : mul2(m23, N[e]));
 }
 
-// Tricubic Hermite value and gradient for two feet, streamed over the four x-lines of
-// the cell (B = y corner, C = z corner).  row(B, C, lo, hi) must fill lo[a], hi[a] with
+// Tricubic Hermite value and gradient for two feet, streamed over the four x-lines of the
+// cell (B = y corner, C = z corner) in two groups of data, phi, psi_x, psi_y, phi_xy (G = 0)
+// and psi_z, phi_xz, phi_yz, phi_xyz (G = 1).  row(G, B, C, lo, hi) must fill lo[a], hi[a]
+// with the group's four data at the line's x = k and x = k+1 corners, for both lanes: a
+// group is reduced along x and y before the next one is loaded, so that 16 instead of 32
+// registers hold x-reduced values.  phi is shifted by its value at the cell's first corner
+// (line B = C = 0, x = k), as in hermite2d_pair.  The reduction order is x, then y, then z,
+// as in the sum-factorised form of Sec. 2.3.
+template <class Row>
+__device__ __forceinline__ void hermite3d_pair(const Basis2 &bx, const Basis2 &by, const Basis2 &bz,
+                                               Row row, F2 &H, F2 g[3])
+{
+    F2 R[2], Rx[2], Ry[2], Rz[2], Rzx[2], Rzy[2];
+    F2 base;
+#pragma unroll
+    for (int C = 0; C < 2; ++C) {
+#pragma unroll
+        for (int G = 0; G < 2; ++G) {
+            F2 P[2], Pd[2], Q[2], Qd[2];  // along x: values of the group's two x-pairs and derivatives
+#pragma unroll
+            for (int B = 0; B < 2; ++B) {
+                F2 lo[4], hi[4];
+                row(G, B, C, lo, hi);
+                if (G == 0) {
+                    if (B == 0 && C == 0) {
+                        base = lo[0];
+                        const F2 p1 = sub2(hi[0], base);
+                        P[B] = hval2z(bx, p1, lo[1], hi[1]);
+                        Pd[B] = hder2z(bx, p1, lo[1], hi[1]);
+                    } else {
+                        const F2 p0 = sub2(lo[0], base), p1 = sub2(hi[0], base);
+                        P[B] = hval2(bx, p0, p1, lo[1], hi[1]);
+                        Pd[B] = hder2(bx, p0, p1, lo[1], hi[1]);
+                    }
+                } else {
+                    P[B] = hval2(bx, lo[0], hi[0], lo[1], hi[1]);
+                    Pd[B] = hder2(bx, lo[0], hi[0], lo[1], hi[1]);
+                }
+                Q[B] = hval2(bx, lo[2], hi[2], lo[3], hi[3]);
+                Qd[B] = hder2(bx, lo[2], hi[2], lo[3], hi[3]);
+            }
+            (G == 0 ? R : Rz)[C] = hval2(by, P[0], P[1], Q[0], Q[1]);
+            (G == 0 ? Ry : Rzy)[C] = hder2(by, P[0], P[1], Q[0], Q[1]);
+            (G == 0 ? Rx : Rzx)[C] = hval2(by, Pd[0], Pd[1], Qd[0], Qd[1]);
+        }
+    }
+    H = add2(base, hval2(bz, R[0], R[1], Rz[0], Rz[1]));
+    g[2] = hder2(bz, R[0], R[1], Rz[0], Rz[1]);
+    g[0] = hval2(bz, Rx[0], Rx[1], Rzx[0], Rzx[1]);
+    g[1] = hval2(bz, Ry[0], Ry[1], Rzy[0], Rzy[1]);
+}
+
+// The same streamed over whole lines, all eight data of a line at once: for stored mixed
+// derivatives, whose loads leave the registers for it (256^3 deformation step kernel 289 us
+// against 293 in groups; feet outside the tile 1 to 2 % more).  row(B, C, lo, hi) must fill lo[a], hi[a] with
 // plane a (0 phi, 1 x, 2 y, 3 z, 4 xy, 5 xz, 6 yz, 7 xyz) at the line's x = k and x = k+1
 // corners, for both lanes.  phi is shifted by its value at the cell's first corner (line
 // B = C = 0, x = k), as in hermite2d_pair.  The reduction order is x, then y, then z, as
@@ -473,7 +526,7 @@ __device__ __forceinline__ XRed2 xreduce2(const Basis2 &bx, const F2 lo[8], cons
 }
 
 template <class Row>
-__device__ __forceinline__ void hermite3d_pair(const Basis2 &bx, const Basis2 &by, const Basis2 &bz,
+__device__ __forceinline__ void hermite3d_lines(const Basis2 &bx, const Basis2 &by, const Basis2 &bz,
                                                Row row, F2 &H, F2 g[3])
 {
     F2 R[2], Rx[2], Ry[2], Rz[2], Rzx[2], Rzy[2];
@@ -503,6 +556,12 @@ __device__ __forceinline__ void hermite3d_pair(const Basis2 &bx, const Basis2 &b
     g[2] = hder2(bz, R[0], R[1], Rz[0], Rz[1]);
     g[0] = hval2(bz, Rx[0], Rx[1], Rzx[0], Rzx[1]);
     g[1] = hval2(bz, Ry[0], Ry[1], Rzy[0], Rzy[1]);
+}
+
+// Planes of the groups' data: entry a of group G.
+__device__ __forceinline__ constexpr int group_plane(int G, int a)
+{
+    return G == 0 ? (a < 3 ? a : 4) : (a == 0 ? 3 : 4 + a);
 }
 
 }  // namespace gals

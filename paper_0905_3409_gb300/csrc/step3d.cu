@@ -9,6 +9,7 @@
 // from psi windows around the cell (COMPACT) with the same stencils.
 #include "step3d_common.cuh"
 
+
 namespace gals {
 
 namespace {
@@ -17,38 +18,85 @@ using namespace t3;
 
 // Output tile per block: TX x TY nodes in x, y and TZ in z (each thread walks TZ nodes in z).
 constexpr int TX = 32, TY = 4, TZ = 4;
-constexpr int HX = 4, HZ = 1;          // halo (x rounded to 16 bytes for TMA)
+constexpr int HX = 4;                  // halo (x rounded to 16 bytes for TMA)
 template <int CR> struct Tile3 {
     // psi_z y-window needs one more row (CROSS_RECON); CROSS_CELL shares that tile's map
+    static constexpr int HZ = 1;
     static constexpr int HY = CR == CROSS_PLANE ? 1 : 2;
     static constexpr int NP = CR == CROSS_PLANE ? 8 : 4;
     static constexpr int W = TX + 2 * HX, H = TY + 2 * HY, D = TZ + 2 * HZ;
     static constexpr int PS = W * H * D;
     static constexpr int BYTES = NP * PS * 4;
+    // CROSS_RECON: phi_yz of the staged nodes is a fifth plane behind them
+    static constexpr int SMEM = BYTES + (CR == CROSS_RECON ? PS * 4 : 0);
 };
+
+// phi_yz = Dy psi_z at every staged node of the rows a foot's cell can use, four nodes of a row
+// at a time (approach A with one-sided ends at the box; nodes outside it hold anything).
+__device__ __forceinline__ void stage_yz(float *tile, const Geom &g, int y0)
+{
+    using T = Tile3<CROSS_RECON>;
+    // a thread keeps its place in the level: rows 1 .. H - 2 of the tile, Q quadruples each
+    constexpr int Q = T::W / 4, R = T::H - 2, N = Q * R, L = TX * TY / N;
+    static_assert(T::W % 4 == 0 && L >= 1, "rows of whole quadruples, a level per pass or more");
+    const int tid = threadIdx.x + TX * threadIdx.y;
+    if (tid >= L * N) return;
+    const int q = tid % Q, r = tid / Q % R + 1, j = y0 - T::HY + r;
+    for (int z = tid / N; z < T::D; z += L) {
+        const int o = (z * T::H + r) * T::W + 4 * q;
+        const float4 *p = reinterpret_cast<const float4 *>(tile + 3 * T::PS + o);
+        constexpr int S = T::W / 4;             // a row further
+        float4 v;
+        if (j == 0) {
+            const float4 a = p[0], b = p[S], c = p[2 * S];
+            v = make_float4(dfirst(a.x, b.x, c.x, g.i2h1), dfirst(a.y, b.y, c.y, g.i2h1),
+                            dfirst(a.z, b.z, c.z, g.i2h1), dfirst(a.w, b.w, c.w, g.i2h1));
+        } else if (j == g.n1 - 1) {
+            const float4 a = p[0], b = p[-S], c = p[-2 * S];
+            v = make_float4(dlast(a.x, b.x, c.x, g.i2h1), dlast(a.y, b.y, c.y, g.i2h1),
+                            dlast(a.z, b.z, c.z, g.i2h1), dlast(a.w, b.w, c.w, g.i2h1));
+        } else {
+            const float4 a = p[S], b = p[-S];
+            v = make_float4(dcentral(a.x, b.x, g.i2h1), dcentral(a.y, b.y, g.i2h1), dcentral(a.z, b.z, g.i2h1),
+                            dcentral(a.w, b.w, g.i2h1));
+        }
+        *reinterpret_cast<float4 *>(tile + 4 * T::PS + o) = v;
+    }
+}
 
 // Two nodes per thread, (i, j, kz) and (i, j, kz+1), in paired FP32: trace with the 3x3
 // Jacobian, cell location, tricubic Hermite value and gradient from the staged tile,
 // phi+ = H and psi+ = J^T grad H.  Feet whose cell data lie outside the staged tile
 // (large CFL) read global memory instead.
-// FULL layout: at most 128 registers (4 blocks per SM; a few words spill), measured faster
-// than 166 registers at 3 blocks per SM.
+// At most 128 registers (4 blocks per SM; a few words spill), measured faster than 166
+// registers at 3 blocks per SM.
+// CROSS_RECON (COMPACT, and FULL between the steps of a run where step_launch chooses it)
+// stages phi and psi only: phi_yz is differenced once per staged node into shared memory and
+// the x-differences are taken, both feet at once, as a cell's lines are read.  It replaces
+// the reconstruction pass (66 us of a 256^3 step) by 115 instructions per node; us per step,
+// against the windows of 16 psi_z per line it used to rebuild phi_yz from / FULL's two
+// passes: 256^3 deformation 344 against 447 / 351, rotation 306 against 406 / 311, 101^3
+// deformation 33.2 against 39.8 / 37.4.  Tiles of 2, 6 or 8 levels (363, 354, 356) and a halo
+// of two cells (397) were slower, as was a branch for the one-sided ends per difference (373).
 template <int TR, int VK, int CR>
-__global__ void __launch_bounds__(TX *TY, CR == CROSS_PLANE ? 4 : 1)
+__global__ void __launch_bounds__(TX *TY, CR == CROSS_CELL ? 1 : 4)
 k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParams vp,
          const StageCoef *__restrict__ coef, float dt, const __grid_constant__ CUtensorMap tmap,
-         int *__restrict__ err, int zt0)
+         int *__restrict__ err, int zlo)
 {
     using T = Tile3<CR>;
     extern __shared__ __align__(128) float tile[];
     __shared__ __align__(8) uint64_t bar;
+    // CROSS_RECON keeps the Jacobian here while the interpolant is evaluated (18 registers)
+    constexpr bool JS = CR == CROSS_RECON && TR != TR_HEUN && VK == VK_DEFORM3D;
+    __shared__ F2 Jsh[JS ? 9 : 1][JS ? TX * TY : 1];
     const int tid = threadIdx.x + TX * threadIdx.y;
-    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = (blockIdx.z + zt0) * TZ;
+    const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = zlo + blockIdx.z * TZ;
     if (tid == 0) mbar_init(&bar, 1);
     __syncthreads();
     if (tid == 0) {
         mbar_arrive_expect_tx(&bar, T::BYTES);
-        tma_load_4d(tile, &tmap, x0 - HX, y0 - T::HY, z0 - HZ, 0, &bar);
+        tma_load_4d(tile, &tmap, x0 - HX, y0 - T::HY, z0 - T::HZ, 0, &bar);
     }
     const StageCoef &sc = *coef;
     // threads past a ragged edge trace a clamped node and store nothing
@@ -74,8 +122,16 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
                 }
                 return;
             }
+            if (CR == CROSS_RECON) {
+                stage_yz(tile, g, y0);
+                __syncthreads();
+            }
         }
         trace3d_pair<TR, VK>(stage1_pair<VK>(vp, sc, pre, X, Y, Z), vp, sc, X, Y, Z, dt, d, J);
+
+        if (JS)
+#pragma unroll
+            for (int e = 0; e < 9; ++e) Jsh[e][tid] = J[e];
 
         int k0, l0, m0, k1, l1, m1;
         float xi0, eta0, zeta0, xi1, eta1, zeta1;
@@ -91,13 +147,13 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
 
         // a cell is served from the tile if every value its line reads is staged
         auto in_tile = [&](int k, int l, int m) {
-            const int tx = k - x0 + HX, ty = l - y0 + T::HY, tz = m - z0 + HZ;
+            const int tx = k - x0 + HX, ty = l - y0 + T::HY, tz = m - z0 + T::HZ;
             return CR != CROSS_RECON
                 ? (tx >= 0 && tx <= T::W - 2 && ty >= 0 && ty <= T::H - 2 && tz >= 0 && tz <= T::D - 2)
                 : (tx >= 1 && tx <= T::W - 3 && ty >= 1 && ty <= T::H - 3 && tz >= 0 && tz <= T::D - 2);
         };
         auto lds = [&](int a, int zz, int yy, int xx) {
-            return tile[GALS_CHK(g, a * T::PS + ((zz - z0 + HZ) * T::H + yy - y0 + T::HY) * T::W + xx - x0 + HX,
+            return tile[GALS_CHK(g, a * T::PS + ((zz - z0 + T::HZ) * T::H + yy - y0 + T::HY) * T::W + xx - x0 + HX,
                                  T::NP * T::PS)];
         };
         auto ldg = [&](int a, int zz, int yy, int xx) {
@@ -123,18 +179,89 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
                 }
             cross_cell3d([&](int v, int a) { return q0[v][a]; }, g.ih0, g.ih1, g.ih2, c0);
             cross_cell3d([&](int v, int a) { return q1[v][a]; }, g.ih0, g.ih1, g.ih2, c1);
-            hermite3d_pair(bx, by, bz, [&](int B, int C, F2 lo[8], F2 hi[8]) {
+            hermite3d_pair(bx, by, bz, [&](int G, int B, int C, F2 lo[4], F2 hi[4]) {
                 const int v = 2 * B + 4 * C;
 #pragma unroll
                 for (int a = 0; a < 4; ++a) {
-                    lo[a] = make_float2(q0[v][a], q1[v][a]);
-                    hi[a] = make_float2(q0[v + 1][a], q1[v + 1][a]);
-                    lo[4 + a] = make_float2(c0[v][a], c1[v][a]);
-                    hi[4 + a] = make_float2(c0[v + 1][a], c1[v + 1][a]);
+                    const int p = group_plane(G, a), e = p < 4 ? p : p - 4;
+                    lo[a] = p < 4 ? make_float2(q0[v][e], q1[v][e]) : make_float2(c0[v][e], c1[v][e]);
+                    hi[a] = p < 4 ? make_float2(q0[v + 1][e], q1[v + 1][e]) : make_float2(c0[v + 1][e], c1[v + 1][e]);
                 }
             }, H, gr);
+        } else if (CR == CROSS_RECON && in0 && in1) {
+            // phi_xy, phi_xz, phi_xyz of the cell's corners by x-differences of psi_y, psi_z and
+            // the staged phi_yz, both feet at once; one-sided where the cell touches the box
+            const float *p0 = tile + (((m0 - z0 + T::HZ) * T::H + l0 - y0 + T::HY) * T::W + k0 - x0 + HX);
+            const float *p1 = tile + (((m1 - z0 + T::HZ) * T::H + l1 - y0 + T::HY) * T::W + k1 - x0 + HX);
+#ifdef GALS_CHECKED
+            // the reads below: planes 0 .. 4, rows and levels up to one further, columns -1 .. 2
+            p0 = tile + 1 + GALS_CHK(g, (int)(p0 - tile) - 1, T::PS - (T::H + 1) * T::W - 3);
+            p1 = tile + 1 + GALS_CHK(g, (int)(p1 - tile) - 1, T::PS - (T::H + 1) * T::W - 3);
+#endif
+            // bits: a foot's cell at the first column (1, 2) or the last one (4, 8)
+            const int edge = (k0 == 0) | (k1 == 0) << 1 | (k0 == g.n0 - 2) << 2 | (k1 == g.n0 - 2) << 3;
+            auto line = [&](int G, int B, int C, F2 lo[4], F2 hi[4], bool ends) {
+                const int o = (C * T::H + B) * T::W;
+                auto ld = [&](int a, int q) { return make_float2(p0[a * T::PS + o + q], p1[a * T::PS + o + q]); };
+                // data v and v + 1 of the group from plane a (psi_y, psi_z, phi_yz) and its Dx
+                auto dx = [&](int a, int v) {
+                    const F2 um = ld(a, -1), u0 = ld(a, 0), u1 = ld(a, 1), up = ld(a, 2);
+                    F2 d0 = mul2(sub2(u1, um), bc(g.i2h0)), d1 = mul2(sub2(up, u0), bc(g.i2h0));
+                    if (ends) {
+                        if (edge & 1) d0.x = dfirst(u0.x, u1.x, up.x, g.i2h0);
+                        if (edge & 2) d0.y = dfirst(u0.y, u1.y, up.y, g.i2h0);
+                        if (edge & 4) d1.x = dlast(u1.x, u0.x, um.x, g.i2h0);
+                        if (edge & 8) d1.y = dlast(u1.y, u0.y, um.y, g.i2h0);
+                    }
+                    lo[v] = u0; hi[v] = u1;
+                    lo[v + 1] = d0; hi[v + 1] = d1;
+                };
+                if (G == 0) {
+                    lo[0] = ld(0, 0); hi[0] = ld(0, 1);
+                    lo[1] = ld(1, 0); hi[1] = ld(1, 1);
+                    dx(2, 2);
+                } else {
+                    dx(3, 0);
+                    dx(4, 2);
+                }
+            };
+            // (a branch per difference cost 24 instructions per node)
+            if (__any_sync(__activemask(), edge))
+                hermite3d_pair(bx, by, bz, [&](int G, int B, int C, F2 lo[4], F2 hi[4]) { line(G, B, C, lo, hi, true); }, H, gr);
+            else
+                hermite3d_pair(bx, by, bz, [&](int G, int B, int C, F2 lo[4], F2 hi[4]) { line(G, B, C, lo, hi, false); }, H, gr);
+        } else if (CR == CROSS_RECON) {
+            // a foot outside the tile: both from global memory, one at a time (both lanes the same
+            // foot), so that this path's windows do not set the kernel's registers
+#pragma unroll 1
+            for (int e = 0; e < 2; ++e) {
+                const int k = e ? k1 : k0, l = e ? l1 : l0, m = e ? m1 : m0;
+                auto dup = [&](const F2 &v) { return bc(e ? v.y : v.x); };
+                const Basis2 ex{dup(bx.S), dup(bx.dS), dup(bx.hG0), dup(bx.hG1), dup(bx.dG0), dup(bx.dG1)};
+                const Basis2 ey{dup(by.S), dup(by.dS), dup(by.hG0), dup(by.hG1), dup(by.dG0), dup(by.dG1)};
+                const Basis2 ez{dup(bz.S), dup(bz.dS), dup(bz.hG0), dup(bz.hG1), dup(bz.dG0), dup(bz.dG1)};
+                F2 He, ge[3];
+                hermite3d_pair(ex, ey, ez, [&](int G, int B, int C, F2 lo[4], F2 hi[4]) {
+                    float a0[8], b0[8];
+                    cell_line<CR>(ldg, g, k, l, m, B, C, a0, b0);
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        lo[a] = bc(a0[group_plane(G, a)]);
+                        hi[a] = bc(b0[group_plane(G, a)]);
+                    }
+                }, He, ge);
+                if (e) {
+                    H.y = He.y;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) gr[a].y = ge[a].y;
+                } else {
+                    H = He;
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) gr[a] = ge[a];
+                }
+            }
         } else if (in0 && in1) {
-            hermite3d_pair(bx, by, bz, [&](int B, int C, F2 lo[8], F2 hi[8]) {
+            hermite3d_lines(bx, by, bz, [&](int B, int C, F2 lo[8], F2 hi[8]) {
                 float a0[8], b0[8], a1[8], b1[8];
                 cell_line<CR>(lds, g, k0, l0, m0, B, C, a0, b0);
                 cell_line<CR>(lds, g, k1, l1, m1, B, C, a1, b1);
@@ -147,7 +274,7 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
         } else {
             auto ld0 = [&](int a, int zz, int yy, int xx) { return in0 ? lds(a, zz, yy, xx) : ldg(a, zz, yy, xx); };
             auto ld1 = [&](int a, int zz, int yy, int xx) { return in1 ? lds(a, zz, yy, xx) : ldg(a, zz, yy, xx); };
-            hermite3d_pair(bx, by, bz, [&](int B, int C, F2 lo[8], F2 hi[8]) {
+            hermite3d_lines(bx, by, bz, [&](int B, int C, F2 lo[8], F2 hi[8]) {
                 float a0[8], b0[8], a1[8], b1[8];
                 cell_line<CR>(ld0, g, k0, l0, m0, B, C, a0, b0);
                 cell_line<CR>(ld1, g, k1, l1, m1, B, C, a1, b1);
@@ -166,6 +293,9 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
             const V3p Dn = stage1_pair<VK>(vp, sc, pre, X, Y, Z);
             heun_psi3(Df, Dn, dt, gr, psi);
         } else {
+            if (JS)
+#pragma unroll
+                for (int e = 0; e < 9; ++e) J[e] = Jsh[e][tid];
 #pragma unroll
             for (int a = 0; a < 3; ++a)  // (J^T grad H)_a = sum_b J[b][a] dH/dx_b
                 psi[a] = fma2(J[a], gr[0], fma2(J[3 + a], gr[1], mul2(J[6 + a], gr[2])));
@@ -293,47 +423,47 @@ k_recon3d_tma(float *__restrict__ buf, Geom g, const __grid_constant__ CUtensorM
 }
 
 template <int TR, int VK, int CR>
-cudaError_t launch_t(const StepLaunch &a, cudaStream_t s, int zt0, int nzt)
+cudaError_t launch_t(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
     using T = Tile3<CR>;
     static bool attr_set = false;
     if (!attr_set) {
         cudaError_t e = cudaFuncSetAttribute(k_step3d<TR, VK, CR>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, T::BYTES);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
         if (e != cudaSuccess) return e;
         attr_set = true;
     }
     dim3 block(TX, TY);
-    dim3 grid((a.geom.n0 + TX - 1) / TX, (a.geom.n1 + TY - 1) / TY, nzt);
+    dim3 grid((a.geom.n0 + TX - 1) / TX, (a.geom.n1 + TY - 1) / TY, (z1 - z0 + TZ - 1) / TZ);
     const CUtensorMap &map = *a.tmap[0][CR == CROSS_PLANE];
-    k_step3d<TR, VK, CR><<<grid, block, T::BYTES, s>>>(a.in, a.out, a.geom, a.vp, a.coef,
-                                                      (float)a.dt, map, a.err, zt0);
+    k_step3d<TR, VK, CR><<<grid, block, T::SMEM, s>>>(a.in, a.out, a.geom, a.vp, a.coef,
+                                                      (float)a.dt, map, a.err, z0);
     return cudaGetLastError();
 }
 
 template <int TR, int VK>
-cudaError_t launch_cr(const StepLaunch &a, cudaStream_t s, int zt0, int nzt)
+cudaError_t launch_cr(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
-    if (a.cross_in == CROSS_CELL) return launch_t<TR, VK, CROSS_CELL>(a, s, zt0, nzt);
-    return a.cross_in == CROSS_PLANE ? launch_t<TR, VK, CROSS_PLANE>(a, s, zt0, nzt)
-                                     : launch_t<TR, VK, CROSS_RECON>(a, s, zt0, nzt);
+    if (a.cross_in == CROSS_CELL) return launch_t<TR, VK, CROSS_CELL>(a, s, z0, z1);
+    return a.cross_in == CROSS_PLANE ? launch_t<TR, VK, CROSS_PLANE>(a, s, z0, z1)
+                                     : launch_t<TR, VK, CROSS_RECON>(a, s, z0, z1);
 }
 
 template <int VK>
-cudaError_t launch_tr(const StepLaunch &a, cudaStream_t s, int zt0, int nzt)
+cudaError_t launch_tr(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
-    if (a.trace == TR_HEUN) return launch_cr<TR_HEUN, VK>(a, s, zt0, nzt);
-    return a.trace == TR_EULER ? launch_cr<TR_EULER, VK>(a, s, zt0, nzt)
-                               : launch_cr<TR_RK3, VK>(a, s, zt0, nzt);
+    if (a.trace == TR_HEUN) return launch_cr<TR_HEUN, VK>(a, s, z0, z1);
+    return a.trace == TR_EULER ? launch_cr<TR_EULER, VK>(a, s, z0, z1)
+                               : launch_cr<TR_RK3, VK>(a, s, z0, z1);
 }
 
-// step kernel over the z-tiles [zt0, zt0 + nzt)
-cudaError_t launch_step_tiles(const StepLaunch &a, cudaStream_t s, int zt0, int nzt)
+// step kernel over the z-levels [z0, z1)
+cudaError_t launch_step_tiles(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
     switch (a.vp.kind) {
-    case VK_CONST: return launch_tr<VK_CONST>(a, s, zt0, nzt);
-    case VK_ROTATION: return launch_tr<VK_ROTATION>(a, s, zt0, nzt);
-    case VK_DEFORM3D: return launch_tr<VK_DEFORM3D>(a, s, zt0, nzt);
+    case VK_CONST: return launch_tr<VK_CONST>(a, s, z0, z1);
+    case VK_ROTATION: return launch_tr<VK_ROTATION>(a, s, z0, z1);
+    case VK_DEFORM3D: return launch_tr<VK_DEFORM3D>(a, s, z0, z1);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -355,7 +485,7 @@ cudaError_t launch_step3d(const StepLaunch &a, cudaStream_t s)
     static_assert(TZ == 4 && QZ == 4, "bands are whole tiles of both kernels");
     const int z0 = a.band_lo, z1 = a.band_hi > 0 ? a.band_hi : a.geom.n2;
     if (z1 <= z0) return cudaSuccess;
-    cudaError_t e = launch_step_tiles(a, s, z0 / TZ, (z1 - z0 + TZ - 1) / TZ);
+    cudaError_t e = launch_step_tiles(a, s, z0, z1);
     if (e != cudaSuccess || !a.write_cross) return e;
     return launch_recon_slabs(a, s, z0 / QZ, (z1 - z0 + QZ - 1) / QZ);
 }
