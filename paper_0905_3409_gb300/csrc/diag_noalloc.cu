@@ -152,7 +152,9 @@ gals_status gals_diagnostics_noalloc(int dim, const int *n, const double *lo, co
     cudaError_t e = scratch_address(&sc);
     if (e != cudaSuccess) return nfail(GALS_ERR_CUDA, cudaGetErrorString(e));
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    const int nparts = (int)((nodes + kNodesPerPartial - 1) / kNodesPerPartial);
+    // a block per partial: at least one per 1024 nodes up to the default number of blocks
+    const int nparts = (int)std::max<int64_t>((nodes + kNodesPerPartial - 1) / kNodesPerPartial,
+                                              std::min<int64_t>((nodes + 1023) / 1024, diag_partials_needed()));
     // launch_diag_with clears the counters first: the scratch keeps the previous call's
     // contents
     e = launch_diag_with(dim, G, state, reference, q, &sc->counters, sc->partials, nparts, s);
