@@ -285,7 +285,9 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
 {
     int cur = g->cur;
     launches = (vp.kind == VK_WAVES2D ? 2 : 1) + 1;  // coefficients (+ wave amplitudes), clock
-    cudaError_t ce = launch_coef_table(g->coef, vp, g->t_dev, dt, nsteps, g->stream);
+    // a plain chain of kernels on one stream: each launched as the dependent of the one before
+    const bool chain = !(bands && bands->n >= 2) && !run && trace != GALS_TRACE_SURROGATE;
+    cudaError_t ce = launch_coef_table(g->coef, vp, g->t_dev, dt, nsteps, g->stream, chain);
     if (ce != cudaSuccess) return ce;
     if (bands && bands->n >= 2) {
         // fork the band streams off the grid stream, chain each band on its two neighbours'
@@ -355,12 +357,13 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
             a.vp.given_plane = g->geom.plane;
             ++launches;
         }
+        a.dependent = chain;
         cudaError_t e = g->dim == 2 ? launch_step2d(a, g->stream) : launch_step3d(a, g->stream);
         if (e != cudaSuccess) return e;
         launches += (g->dim == 3 && a.write_cross) ? 2 : 1;  // 3D FULL: step + reconstruction
         cur ^= 1;
     }
-    return launch_advance_time(g->t_dev, nsteps, dt, g->stream);
+    return launch_advance_time(g->t_dev, nsteps, dt, g->stream, chain);
 }
 
 // A run on a small 2D grid: coefficients, one cluster launch, clock.

@@ -9,6 +9,27 @@
 
 namespace gals {
 
+// Launch `kern` on s; dependent: as a programmatic dependent of the kernel before it (see
+// pdl_wait), so that its launch overlaps that kernel.  For chains of small kernels, us per
+// step: a 64^2 step called by itself (coefficients, step, clock) 11.5 -> 8.4, 3D graphs of
+// 20^3 7 -> 4.7, 64 x 60 x 50 9.2 -> 8.0; steps of many waves of blocks lose nothing.
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, bool dependent,
+                          const A &...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = dependent ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 struct StepLaunch {
     const float *in;     // state at t (all planes, plane stride geom.plane)
     float *out;          // state at t + dt
@@ -27,6 +48,7 @@ struct StepLaunch {
     // the band of nodes to update along the last axis (2D rows, 3D z-levels), [lo, hi);
     // hi == 0: all.  lo must be a multiple of band_unit(dim), hi too unless it is n.
     int band_lo, band_hi;
+    bool dependent;      // launch_kernel's
 };
 
 // Persistent 2D time loop (FULL layout, approach A): nsteps steps from buffer cur in one
@@ -98,9 +120,9 @@ cudaError_t launch_step3d(const StepLaunch &a, cudaStream_t s);
 cudaError_t launch_recon(int dim, const Geom &g, float *buf, cudaStream_t s);
 // table[s] = stage coefficients of step s (t = t_dev[0] + s*dt), s < nsteps
 cudaError_t launch_coef_table(StageCoef *table, const VelParams &vp, const double *t_dev,
-                              double dt, int nsteps, cudaStream_t s);
+                              double dt, int nsteps, cudaStream_t s, bool dependent = false);
 // t_dev[0] += nsteps * dt
-cudaError_t launch_advance_time(double *t_dev, int nsteps, double dt, cudaStream_t s);
+cudaError_t launch_advance_time(double *t_dev, int nsteps, double dt, cudaStream_t s, bool dependent = false);
 // the device clock set to t, in stream order (no host staging, the caller does not block)
 cudaError_t launch_set_time(double *t_dev, double t, cudaStream_t s);
 // Velocity kinds supported per dimension.

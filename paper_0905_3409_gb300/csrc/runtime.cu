@@ -1,6 +1,7 @@
 // runtime.cu -- small launchers shared by the C ABI: approach-A reconstruction dispatch,
 // the device clock update and the velocity/dimension support table.
 #include "gals_internal.h"
+#include "tma.cuh"
 
 namespace gals {
 
@@ -15,6 +16,8 @@ cudaError_t launch_recon(int dim, const Geom &g, float *buf, cudaStream_t s)
 namespace {
 __global__ void k_advance_time(double *t, int nsteps, double dt)
 {
+    pdl_wait();
+    pdl_release();
     if (threadIdx.x == 0 && blockIdx.x == 0) t[0] = t[0] + (double)nsteps * dt;
 }
 
@@ -33,6 +36,8 @@ k_coef_table(StageCoef *table, const __grid_constant__ VelParams vp, const doubl
 {
     __shared__ double term[kCoefWarps][3 * kMaxModes];
     const int w = threadIdx.x >> 5, k = blockIdx.x * kCoefWarps + w;
+    pdl_wait();
+    pdl_release();
     if (k >= nsteps) return;
     stage_coef_warp(vp, t_dev[0] + (double)k * dt, dt, table[k], term[w]);
     if (vp.kind == VK_WAVES2D && (threadIdx.x & 31) == 3) table[k].wamp = vp.wamp + (size_t)k * 3 * vp.nwaves;
@@ -40,10 +45,12 @@ k_coef_table(StageCoef *table, const __grid_constant__ VelParams vp, const doubl
 
 // WAVES2D amplitudes of the call's steps: wamp[(k 3 + s) M + m] = a_m cos(2 pi (n_m t_s + chi_m'))
 // at the stage times t_s (t + dt, t, t + dt/2) of step k, the phase reduced in FP64.
-__global__ void k_wave_amp(VelParams vp, const double *t_dev, double dt, int nsteps)
+__global__ void k_wave_amp(const __grid_constant__ VelParams vp, const double *t_dev, double dt, int nsteps)
 {
     const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int M = vp.nwaves;
+    pdl_wait();
+    pdl_release();
     if (e >= (int64_t)nsteps * 3 * M) return;
     const int m = (int)(e % M), s = (int)((e / M) % 3), k = (int)(e / (3 * M));
     const double t = t_dev[0] + (double)k * dt;
@@ -56,22 +63,21 @@ __global__ void k_wave_amp(VelParams vp, const double *t_dev, double dt, int nst
 }  // namespace
 
 cudaError_t launch_coef_table(StageCoef *table, const VelParams &vp, const double *t_dev,
-                              double dt, int nsteps, cudaStream_t s)
+                              double dt, int nsteps, cudaStream_t s, bool dependent)
 {
     if (vp.kind == VK_WAVES2D) {
         const int64_t n = (int64_t)nsteps * 3 * vp.nwaves;
-        k_wave_amp<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(vp, t_dev, dt, nsteps);
-        cudaError_t e = cudaGetLastError();
+        cudaError_t e = launch_kernel(k_wave_amp, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, s, dependent, vp,
+                                      t_dev, dt, nsteps);
         if (e != cudaSuccess) return e;
     }
-    k_coef_table<<<(nsteps + kCoefWarps - 1) / kCoefWarps, 32 * kCoefWarps, 0, s>>>(table, vp, t_dev, dt, nsteps);
-    return cudaGetLastError();
+    return launch_kernel(k_coef_table, dim3((nsteps + kCoefWarps - 1) / kCoefWarps), dim3(32 * kCoefWarps), 0, s,
+                         dependent, table, vp, t_dev, dt, nsteps);
 }
 
-cudaError_t launch_advance_time(double *t_dev, int nsteps, double dt, cudaStream_t s)
+cudaError_t launch_advance_time(double *t_dev, int nsteps, double dt, cudaStream_t s, bool dependent)
 {
-    k_advance_time<<<1, 32, 0, s>>>(t_dev, nsteps, dt);
-    return cudaGetLastError();
+    return launch_kernel(k_advance_time, dim3(1), dim3(32), 0, s, dependent, t_dev, nsteps, dt);
 }
 
 cudaError_t launch_set_time(double *t_dev, double t, cudaStream_t s)

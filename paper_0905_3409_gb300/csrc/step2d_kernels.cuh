@@ -60,6 +60,7 @@ k_step2d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
     extern __shared__ __align__(128) float tile[];
     __shared__ __align__(16) Smem<TY, WC> sm;
     if (threadIdx.x == 0) mbar_init(&sm.bar, 1);
+    pdl_wait();
     __syncthreads();
     tile_step2d<TY, TR, VK, CR, WC, HYT, false, TWS, overlapped<WC>()>(
         in, out, g, vp, coef, dt, &tmap, err, blockIdx.x * tile_stride<WC>(), row0 + blockIdx.y * TY, tile, sm, 0);
@@ -75,6 +76,7 @@ k_walk2d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
     extern __shared__ __align__(128) float tile[];
     __shared__ __align__(16) WalkSmem<TY> sm;
     if (threadIdx.x == 0) mbar_init(&sm.bar, 1);
+    pdl_wait();
     __syncthreads();
     tile_walk2d<TY, TR, VK, CR, HYT, TWS>(in, out, g, vp, coef, dt, &tmap, err, blockIdx.x * TX,
                                           row0 + blockIdx.y * TY, row_end, tile, sm, 0);
@@ -219,10 +221,11 @@ cudaError_t launch_ty(const StepLaunch &a, cudaStream_t s)
     const dim3 grid((a.geom.n0 + tile_stride<WC>() - 1) / tile_stride<WC>(), (row1 - row0 + TYT - 1) / TYT);
     const CUtensorMap &map = *a.tmap[TYT == TYS][NP - 3];
     if constexpr (!walked<TYT, VK, CR, WC>())
-        k_step2d<TYT, TR, VK, CR, WC><<<grid, TX, bytes, s>>>(a.in, a.out, a.geom, a.vp, a.coef, (float)a.dt, map, a.err, row0);
+        return launch_kernel(k_step2d<TYT, TR, VK, CR, WC>, grid, dim3(TX), bytes, s, a.dependent, a.in, a.out, a.geom,
+                             a.vp, a.coef, (float)a.dt, map, a.err, row0);
     else
-        k_walk2d<TYT, TR, VK, CR><<<grid, TX, bytes, s>>>(a.in, a.out, a.geom, a.vp, a.coef, (float)a.dt, map, a.err, row0, row1);
-    return cudaGetLastError();
+        return launch_kernel(k_walk2d<TYT, TR, VK, CR>, grid, dim3(TX), bytes, s, a.dependent, a.in, a.out, a.geom,
+                             a.vp, a.coef, (float)a.dt, map, a.err, row0, row1);
 }
 
 template <int TR, int VK, int CR, int WC>

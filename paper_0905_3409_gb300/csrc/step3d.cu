@@ -93,6 +93,7 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
     const int tid = threadIdx.x + TX * threadIdx.y;
     const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = zlo + blockIdx.z * TZ;
     if (tid == 0) mbar_init(&bar, 1);
+    pdl_wait();
     __syncthreads();
     if (tid == 0) {
         mbar_arrive_expect_tx(&bar, T::BYTES);
@@ -127,6 +128,7 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
                 __syncthreads();
             }
         }
+        if (kz + 2 >= zend) pdl_release();
         trace3d_pair<TR, VK>(stage1_pair<VK>(vp, sc, pre, X, Y, Z), vp, sc, X, Y, Z, dt, d, J);
 
         if (JS)
@@ -376,6 +378,7 @@ k_recon3d_tma(float *__restrict__ buf, Geom g, const __grid_constant__ CUtensorM
     const int x0 = blockIdx.x * QX, y0 = blockIdx.y * QY;
     const int z0 = (zq0 + (int)gridDim.z - 1 - (int)blockIdx.z) * QZ;
     if (tid == 0) mbar_init(&bar, 1);
+    pdl_wait();
     __syncthreads();
     if (tid == 0) {
         mbar_arrive_expect_tx(&bar, (uint32_t)sizeof(t));
@@ -436,9 +439,8 @@ cudaError_t launch_t(const StepLaunch &a, cudaStream_t s, int z0, int z1)
     dim3 block(TX, TY);
     dim3 grid((a.geom.n0 + TX - 1) / TX, (a.geom.n1 + TY - 1) / TY, (z1 - z0 + TZ - 1) / TZ);
     const CUtensorMap &map = *a.tmap[0][CR == CROSS_PLANE];
-    k_step3d<TR, VK, CR><<<grid, block, T::SMEM, s>>>(a.in, a.out, a.geom, a.vp, a.coef,
-                                                      (float)a.dt, map, a.err, z0);
-    return cudaGetLastError();
+    return launch_kernel(k_step3d<TR, VK, CR>, grid, block, T::SMEM, s, a.dependent, a.in, a.out, a.geom, a.vp, a.coef,
+                         (float)a.dt, map, a.err, z0);
 }
 
 template <int TR, int VK>
@@ -472,8 +474,7 @@ cudaError_t launch_step_tiles(const StepLaunch &a, cudaStream_t s, int z0, int z
 cudaError_t launch_recon_slabs(const StepLaunch &a, cudaStream_t s, int zq0, int nzq)
 {
     dim3 grid((a.geom.n0 + QX - 1) / QX, (a.geom.n1 + QY - 1) / QY, nzq);
-    k_recon3d_tma<<<grid, dim3(QX, QY), 0, s>>>(a.out, a.geom, *a.tmap_cross, a.err, zq0);
-    return cudaGetLastError();
+    return launch_kernel(k_recon3d_tma, grid, dim3(QX, QY), 0, s, a.dependent, a.out, a.geom, *a.tmap_cross, a.err, zq0);
 }
 
 }  // namespace

@@ -15,6 +15,15 @@ namespace gals {
 constexpr int kErrTmaTimeout = 1;
 constexpr uint32_t kWaitLimit = 1u << 24;  // try_wait polls before a wait counts as lost
 
+// Programmatic dependent launch: wait until the kernel before this one in the stream has
+// finished and its writes are visible (at once if it was not launched as its dependent), and
+// let the one after it be placed while this one runs.  Every kernel that is launched as a
+// dependent waits before its first read or write of global memory.  The step kernels release
+// late (3D: at a thread's last pair of nodes) or at their end: blocks of the next step placed
+// at their start took the places unevenly (64 x 60 x 50: 9.6 us per step against 8.0).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void *p)
 {
     return (uint32_t)__cvta_generic_to_shared(p);
