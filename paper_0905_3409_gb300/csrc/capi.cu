@@ -18,6 +18,7 @@
 #include "../../include/gals.h"
 #include "gals_internal.h"
 #include "capi_internal.h"
+#include "copy_planes.h"
 
 using namespace gals;
 
@@ -71,6 +72,7 @@ struct gals_grid {
     char *pt_buf = nullptr;       // gals_eval_points: device staging of host points / results
     size_t pt_cap = 0;
     int *err_dev = nullptr;       // device error word written by kernels (bounded waits)
+    int *err_host = nullptr;      // its page-locked copy, filled on the stream before a wait
     StageCoef *coef = nullptr;    // per-step stage coefficients of the current call
     int coef_cap = 0;
     DiagOut *diag_dev = nullptr;
@@ -512,6 +514,7 @@ gals_status gals_create_grid(const gals_grid_desc *d, gals_grid **out)
     }
     if ((e = cudaMalloc(&g->t_dev, sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&g->err_dev, sizeof(int))) != cudaSuccess ||
+        (e = cudaMallocHost(&g->err_host, sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc(&g->diag_dev, sizeof(DiagOut))) != cudaSuccess ||
         (e = cudaMalloc(&g->diag_partials, sizeof(double) * diag_partials_needed())) != cudaSuccess) {
         gals_status st = cuda_fail(nullptr, e, "cudaMalloc(aux)");
@@ -574,6 +577,7 @@ gals_status gals_destroy_grid(gals_grid *g)
     for (int b = 0; b < 2; ++b) cudaFree(g->buf[b]);
     cudaFree(g->t_dev);
     cudaFree(g->err_dev);
+    cudaFreeHost(g->err_host);
     cudaFree(g->trace_buf);
     cudaFree(g->pt_buf);
     cudaFree(g->coef);
@@ -626,7 +630,13 @@ gals_status gals_set_state(gals_grid *g, const float *const *fields, int nfields
     const cudaMemcpyKind kind = memspace == GALS_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     float *dst = g->buf[g->cur];
     cudaError_t e;
-    for (int p = 0; p < nfields; ++p) {
+    bool copied = false;
+    if (memspace == GALS_MEM_DEVICE) {
+        const PlaneCopy c{dst, G.plane, G.pitch, g->n[0], (int64_t)rows, const_cast<float *const *>(fields), nfields,
+                          false, nullptr, nullptr};
+        if ((e = copy_planes(c, g->stream, &copied)) != cudaSuccess) return cuda_fail(g, e, "set_state copy");
+    }
+    for (int p = 0; p < nfields && !copied; ++p) {
         e = cudaMemcpy2DAsync(dst + p * G.plane, (size_t)G.pitch * sizeof(float), fields[p], row, row,
                               rows, kind, g->stream);
         if (e != cudaSuccess) return cuda_fail(g, e, "set_state copy");
@@ -819,11 +829,16 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
 }
 
 // After a stream synchronisation: report (and clear) a kernel-side error word.
-static gals_status check_device_error(gals_grid *g)
+// Wait for the grid's stream and report the error word; copied: queued work stores it in
+// err_host already.
+static gals_status wait_and_check(gals_grid *g, const char *what, bool copied = false)
 {
-    int code = 0;
-    cudaError_t e = cudaMemcpy(&code, g->err_dev, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(g, e, "error word");
+    cudaError_t e = cudaSuccess;
+    if (!copied)
+        e = cudaMemcpyAsync(g->err_host, g->err_dev, sizeof(int), cudaMemcpyDeviceToHost, g->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    if (e != cudaSuccess) return cuda_fail(g, e, what);
+    const int code = *(volatile int *)g->err_host;
     if (code == 0) return GALS_OK;
     cudaMemset(g->err_dev, 0, sizeof(int));
     if ((code & 0xff) == kErrBounds)
@@ -837,9 +852,7 @@ gals_status gals_synchronize(gals_grid *g)
 {
     if (!g) return fail(nullptr, GALS_ERR_ARG, "grid is NULL");
     if (cudaError_t je = join_host_steps(g); je != cudaSuccess) return cuda_fail(g, je, "join host steps");
-    cudaError_t e = cudaStreamSynchronize(g->stream);
-    if (e != cudaSuccess) return cuda_fail(g, e, "synchronize");
-    return check_device_error(g);
+    return wait_and_check(g, "synchronize");
 }
 
 static gals_status ensure_cross(gals_grid *g)
@@ -874,13 +887,18 @@ gals_status gals_read_state(gals_grid *g, float *const *fields, int nfields, int
     const size_t rows = (size_t)g->n[1] * g->n[2];
     const cudaMemcpyKind kind = memspace == GALS_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     cudaError_t e;
-    for (int p = 0; p < nfields; ++p) {
+    bool copied = false;
+    if (memspace == GALS_MEM_DEVICE) {
+        const PlaneCopy c{g->buf[g->cur], G.plane, G.pitch, g->n[0], (int64_t)rows, fields, nfields, true,
+                          g->err_dev, g->err_host};
+        if ((e = copy_planes(c, g->stream, &copied)) != cudaSuccess) return cuda_fail(g, e, "read_state copy");
+    }
+    for (int p = 0; p < nfields && !copied; ++p) {
         e = cudaMemcpy2DAsync(fields[p], row, g->buf[g->cur] + p * G.plane, (size_t)G.pitch * sizeof(float),
                               row, rows, kind, g->stream);
         if (e != cudaSuccess) return cuda_fail(g, e, "read_state copy");
     }
-    if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return cuda_fail(g, e, "read_state sync");
-    return check_device_error(g);
+    return wait_and_check(g, "read_state sync", copied);
 }
 
 // gals_step_host and gals_step_host_async: queue the band pipeline; the synchronous form
@@ -1007,7 +1025,7 @@ static gals_status step_host_impl(gals_grid *g, const gals_velocity *v, double d
     g->steps = 1;
     g->cross_explicit = false;
     g->has_state = true;
-    return check_device_error(g);
+    return wait_and_check(g, "error word");
 }
 
 gals_status gals_step_host(gals_grid *g, const gals_velocity *v, double dt, double t0,
@@ -1115,8 +1133,7 @@ gals_status gals_diagnostics(gals_grid *g, const gals_diag_request *req, gals_di
     DiagOut h;
     if ((e = cudaMemcpyAsync(&h, g->diag_dev, sizeof(h), cudaMemcpyDeviceToHost, g->stream)) != cudaSuccess)
         return cuda_fail(g, e, "diagnostics copy");
-    if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return cuda_fail(g, e, "diagnostics sync");
-    if ((st = check_device_error(g)) != GALS_OK) return st;
+    if ((st = wait_and_check(g, "diagnostics sync")) != GALS_OK) return st;
     std::memset(out, 0, sizeof(*out));
     double cell = 1.0;
     int64_t ncell = 1;

@@ -17,6 +17,7 @@
 
 #include "batch_internal.h"
 #include "capi_internal.h"
+#include "copy_planes.h"
 
 using namespace gals;
 
@@ -55,6 +56,7 @@ struct gals_batch {
     StageCoef *coef = nullptr;
     int64_t coef_cap = 0;
     int *err_dev = nullptr;
+    int *err_host = nullptr;               // page-locked copy of the error word
     int cur = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -240,11 +242,16 @@ cudaError_t issue(gals_batch *b, int kind, int nsteps)
     return launch_batch_advance(b->t_dev, b->probs_dev, b->count, nsteps, b->stream);
 }
 
-gals_status check_err(gals_batch *b)
+// Wait for the batch's stream and report the error word; copied: queued work stores it in
+// err_host already.
+gals_status wait_and_check(gals_batch *b, const char *what, bool copied = false)
 {
-    int code = 0;
-    cudaError_t e = cudaMemcpy(&code, b->err_dev, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return bcuda(b, e, "error word");
+    cudaError_t e = cudaSuccess;
+    if (!copied)
+        e = cudaMemcpyAsync(b->err_host, b->err_dev, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) return bcuda(b, e, what);
+    const int code = *(volatile int *)b->err_host;
     if (code == 0) return GALS_OK;
     cudaMemset(b->err_dev, 0, sizeof(int));
     if ((code & 0xff) == kErrBounds)
@@ -332,7 +339,8 @@ gals_status gals_create_batch(const gals_grid_desc *descs, int count, gals_batch
     if ((e = cudaMalloc(&b->probs_dev, sizeof(BatchProb) * count)) != cudaSuccess ||
         (e = cudaMalloc(&b->vps_dev, sizeof(VelParams) * count)) != cudaSuccess ||
         (e = cudaMalloc(&b->t_dev, sizeof(double) * count)) != cudaSuccess ||
-        (e = cudaMalloc(&b->err_dev, sizeof(int))) != cudaSuccess)
+        (e = cudaMalloc(&b->err_dev, sizeof(int))) != cudaSuccess ||
+        (e = cudaMallocHost(&b->err_host, sizeof(int))) != cudaSuccess)
         return bail(e, "cudaMalloc(descriptors)");
     if ((e = cudaMemsetAsync(b->err_dev, 0, sizeof(int), b->stream)) != cudaSuccess) return bail(e, "cudaMemset");
 #ifdef GALS_CHECKED
@@ -432,6 +440,7 @@ gals_status gals_destroy_batch(gals_batch *b)
     cudaFree(b->t_dev);
     cudaFree(b->coef);
     cudaFree(b->err_dev);
+    cudaFreeHost(b->err_host);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
     return GALS_OK;
@@ -453,7 +462,13 @@ gals_status gals_batch_set_state(gals_batch *b, int index, const float *const *f
     const cudaMemcpyKind kind = memspace == GALS_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     float *dst = b->buf[b->cur] + P.off;
     cudaError_t e;
-    for (int p = 0; p < nfields; ++p)
+    bool copied = false;
+    if (memspace == GALS_MEM_DEVICE) {
+        const PlaneCopy c{dst, G.plane, G.pitch, G.n0, G.n1, const_cast<float *const *>(fields), nfields, false,
+                          nullptr, nullptr};
+        if ((e = copy_planes(c, b->stream, &copied)) != cudaSuccess) return bcuda(b, e, "set_state copy");
+    }
+    for (int p = 0; p < nfields && !copied; ++p)
         if ((e = cudaMemcpy2DAsync(dst + p * G.plane, (size_t)G.pitch * 4, fields[p], row, row, G.n1, kind,
                                    b->stream)) != cudaSuccess)
             return bcuda(b, e, "set_state copy");
@@ -530,9 +545,7 @@ gals_status gals_batch_step(gals_batch *b, const gals_velocity *vels, const doub
 gals_status gals_batch_synchronize(gals_batch *b)
 {
     if (!b) return bfail(nullptr, GALS_ERR_ARG, "batch is NULL");
-    cudaError_t e = cudaStreamSynchronize(b->stream);
-    if (e != cudaSuccess) return bcuda(b, e, "synchronize");
-    return check_err(b);
+    return wait_and_check(b, "synchronize");
 }
 
 gals_status gals_batch_read_state(gals_batch *b, int index, float *const *fields, int nfields, int memspace)
@@ -552,12 +565,16 @@ gals_status gals_batch_read_state(gals_batch *b, int index, float *const *fields
         if ((e = launch_recon(2, G, src, b->stream)) != cudaSuccess) return bcuda(b, e, "recon");
     const size_t row = (size_t)G.n0 * sizeof(float);
     const cudaMemcpyKind kind = memspace == GALS_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    for (int p = 0; p < nfields; ++p)
+    bool copied = false;
+    if (memspace == GALS_MEM_DEVICE) {
+        const PlaneCopy c{src, G.plane, G.pitch, G.n0, G.n1, fields, nfields, true, b->err_dev, b->err_host};
+        if ((e = copy_planes(c, b->stream, &copied)) != cudaSuccess) return bcuda(b, e, "read_state copy");
+    }
+    for (int p = 0; p < nfields && !copied; ++p)
         if ((e = cudaMemcpy2DAsync(fields[p], row, src + p * G.plane, (size_t)G.pitch * 4, row, G.n1, kind,
                                    b->stream)) != cudaSuccess)
             return bcuda(b, e, "read_state copy");
-    if ((e = cudaStreamSynchronize(b->stream)) != cudaSuccess) return bcuda(b, e, "read_state sync");
-    return check_err(b);
+    return wait_and_check(b, "read_state sync", copied);
 }
 
 gals_status gals_batch_set_tuning(gals_batch *b, const gals_batch_tuning *t)
@@ -669,7 +686,7 @@ gals_status gals_batch_autotune(gals_batch *b, const gals_velocity *vels, const 
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (e != cudaSuccess) return bcuda(b, e, "autotune launch");
-    if ((st = check_err(b)) != GALS_OK) return st;
+    if ((st = wait_and_check(b, "error word")) != GALS_OK) return st;
     b->tuning = best;
     if (out) *out = best;
     return GALS_OK;
