@@ -13,8 +13,9 @@
 // FP16 pairs.)  Operands use the no-swizzle K-major core-matrix layout: 8 rows
 // x 16 bytes per core matrix, core matrices adjacent in K `lbo` bytes apart and adjacent
 // in M/N 128 bytes apart.  The trace kernel turns the outputs into the foot displacement
-// and the Jacobian of the backward map, checks a few nodes of every tile against the exact
-// RK3 trace (Sec. 5.1) and recomputes the whole tile with RK3 when the check fails.
+// and the Jacobian of the backward map; a fifth warp per group checks a few nodes of every
+// tile against the exact RK3 trace (Sec. 5.1), and the group recomputes the whole tile with
+// RK3 when the check fails.
 #include <cuda_fp16.h>
 
 #include "mlp_internal.h"
@@ -101,7 +102,7 @@ __device__ void block_setup(Smem &sm, const InferParams &ip)
 {
     const uint4 *src = reinterpret_cast<const uint4 *>(ip.w);
     uint4 *dst = reinterpret_cast<uint4 *>(sm.w);
-    for (int e = threadIdx.x; e < (int)(W_TOTAL * 2 / 16); e += NT) dst[e] = src[e];
+    for (int e = threadIdx.x; e < (int)(W_TOTAL * 2 / 16); e += blockDim.x) dst[e] = src[e];
     if (threadIdx.x < NWG) {
         mbar_init(&sm.bar[threadIdx.x], 1);
         sm.fail[threadIdx.x] = 0;
@@ -208,7 +209,7 @@ __device__ bool run_tile(Smem &sm, Wg &w, int *err, float out[8])
             // layer's A operand (K = 128)
             char *arow = reinterpret_cast<char *>(sm.act[g]) + (w.r >> 3) * 128 + (w.r & 7) * 16;
             // one 32-column TMEM load per wait: two per wait held 64 accumulator values live
-            // and pushed the trace kernel past its 168-register cap (spills)
+            // and pushed the trace kernel past its register cap (spills)
             constexpr int NU = 1;
 #pragma unroll 1
             for (int c = 0; c < 4; c += NU) {
@@ -281,100 +282,130 @@ __device__ __forceinline__ uint32_t tile_hash(uint32_t a, uint32_t b)
     return h ^ (h >> 13);
 }
 
-// Surrogate trace of one step over the grid: tile = 128 consecutive nodes of a row; VK
-// is the field of the exact trace the residual check and the fallback run.
+// named barrier id: the tile group arrives (or waits), its checking warp waits (or arrives)
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(GT + 32) : "memory"); }
+__device__ __forceinline__ void pair_arrive(int id)
+{
+    asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(GT + 32) : "memory");
+}
+constexpr int kBarWritten = 1 + NWG, kBarChecked = 1 + 2 * NWG;
+constexpr int NTT = NT + 32 * NWG;  // threads per block of the trace kernel
+
+// Whether one of the tile's sampled nodes is off the exact RK3 trace: warp-wide, the
+// network's values read back from the trace planes.
 template <int VK>
-__global__ void __launch_bounds__(NT, 1)
+__device__ __forceinline__ bool tile_fails(const InferParams &ip, const Geom &g, const VelParams &vp,
+                                           const StageCoef &coef, float dtf, const float *trace, int tile, int tiles_x,
+                                           int kstep, const Check &chk)
+{
+    const int lane = threadIdx.x & 31;
+    const int j = tile / tiles_x, x0 = (tile % tiles_x) * ROWS, width = min(ROWS, g.n0 - x0);
+    const float yy = g.lo1 + (float)j * g.h1;
+    bool bad = false;
+    // a costly field: each node's trace by the whole warp (modes split over the lanes)
+    constexpr bool WARP = VK == VK_WAVES2D;
+    for (int jj = WARP ? 0 : lane; jj < chk.samples; jj += WARP ? 1 : 32) {
+        const int q = (int)(tile_hash((uint32_t)tile, (uint32_t)kstep + 977u * jj) % (uint32_t)width);
+        const float xq = g.lo0 + (float)(x0 + q) * g.h0;
+        float dr[2], Jr[4], m[6];
+        const int64_t o = (int64_t)j * g.pitch + x0 + q;
+#pragma unroll
+        for (int e = 0; e < 6; ++e) m[e] = trace[e * g.plane + o];
+        if (WARP) trace2d_waves_warp(vp, coef, xq, yy, dtf, dr[0], dr[1], Jr);
+        else trace2d<TR_RK3, VK>(vp, coef, xq, yy, dtf, dr[0], dr[1], Jr);
+        const float ex = fmaxf(fabsf(m[0] - dr[0]) * g.ih0, fabsf(m[1] - dr[1]) * g.ih1);
+        float eJ = 0.f;
+        for (int e = 0; e < 4; ++e) eJ = fmaxf(eJ, fabsf(m[2 + e] - Jr[e]));
+        bad = bad || !(ex <= chk.tol_x) || !(eJ <= chk.tol_J);
+    }
+    return __any_sync(0xffffffffu, bad);
+}
+
+// Surrogate trace of one step over the grid: tile = 128 consecutive nodes of a row; VK
+// is the field of the exact trace the residual check and the fallback run.  Latency bounds the
+// kernel (12 warps of network, MUFU and tensor pipes a third busy), and the check of 4 nodes
+// is one long FP32 chain on 4 lanes that used to hold up the tile's other threads: now a
+// fifth warp of the group checks a tile, read back from the trace planes, while the group
+// runs the next one, and the group recomputes a tile that failed one tile later.  2048^2,
+// 16 modes, a whole step: 794 -> 733 us with 4 nodes, 809 -> 766 with 128 nodes a tile (four
+// rounds of the warp), 876 -> 842 where every tile fails; 500^2 70.5 -> 68.
+template <int VK>
+__global__ void __launch_bounds__(NTT, 1)
 k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ coef,
-            const double *__restrict__ t_dev, int kstep, double dt, float *__restrict__ trace,
-            Check chk)
+            const double *__restrict__ t_dev, int kstep, double dt, float *trace, Check chk)
 {
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     block_setup(sm, ip);
-    Wg w = make_wg(sm);
-    bool aborted = false;
-    const double t = t_dev[0] + (double)kstep * dt;
-    const float phase = (float)(t - floor(t));
     const float dtf = (float)dt;
     const int tiles_x = (g.n0 + ROWS - 1) / ROWS;
     const int ntiles = tiles_x * g.n1;
-    // outputs of the tile's rows for the residual check (act[g] is free after the products)
-    float *outs = reinterpret_cast<float *>(sm.act[w.g]);
-    for (int tile = blockIdx.x * NWG + w.g; tile < ntiles; tile += gridDim.x * NWG) {
-        const int j = tile / tiles_x, x0 = (tile % tiles_x) * ROWS;
-        const int i = x0 + w.r;
-        if (w.r == 0) sm.fail[w.g] = 0;
-        {
-            const float x = g.lo0 + (float)min(i, g.n0 - 1) * g.h0, y = g.lo1 + (float)j * g.h1;
-            stage_input(sm, w, 2.f * x - 1.f, 2.f * y - 1.f, 2.f * phase - 1.f);
-        }
-        float y[8];
-        if (!run_tile(sm, w, chk.err, y)) { aborted = true; break; }
-        for (int c = 0; c < OUT; ++c) outs[w.r * 8 + c] = y[c];
-        float d[2], J[4];
-        d[0] = y[0] * ip.scale[0] * g.h0;
-        d[1] = y[1] * ip.scale[1] * g.h1;
-        J[0] = 1.f + dtf * y[2] * ip.scale[2];
-        J[1] = dtf * y[3] * ip.scale[3];
-        J[2] = dtf * y[4] * ip.scale[4];
-        J[3] = 1.f + dtf * y[5] * ip.scale[5];
-        wg_sync(w.g);
-        // residual check of `samples` nodes of the tile against the exact RK3 trace
-        const int width = min(ROWS, g.n0 - x0);
-        if (VK == VK_WAVES2D) {
-            // a costly field: each sampled node's trace by a whole warp of the group
-            // (modes split over the lanes), sample j on warp j mod 4
-            for (int jj = w.r >> 5; jj < chk.samples; jj += GT / 32) {
-                const int q = (int)(tile_hash((uint32_t)tile, (uint32_t)kstep + 977u * jj) % (uint32_t)width);
-                const float *yq = &outs[q * 8];
-                const float xq = g.lo0 + (float)(x0 + q) * g.h0, yy = g.lo1 + (float)j * g.h1;
-                float dr[2], Jr[4];
-                trace2d_waves_warp(vp, *coef, xq, yy, dtf, dr[0], dr[1], Jr);
-                const float ex = fmaxf(fabsf(yq[0] * ip.scale[0] * g.h0 - dr[0]) * g.ih0,
-                                       fabsf(yq[1] * ip.scale[1] * g.h1 - dr[1]) * g.ih1);
-                const float mJ[4] = {1.f + dtf * yq[2] * ip.scale[2], dtf * yq[3] * ip.scale[3],
-                                     dtf * yq[4] * ip.scale[4], 1.f + dtf * yq[5] * ip.scale[5]};
-                float eJ = 0.f;
-                for (int e = 0; e < 4; ++e) eJ = fmaxf(eJ, fabsf(mJ[e] - Jr[e]));
-                if ((w.r & 31) == 0 && (!(ex <= chk.tol_x) || !(eJ <= chk.tol_J))) atomicOr(&sm.fail[w.g], 1);
+    if (threadIdx.x >= NT) {
+        const int gg = (threadIdx.x - NT) >> 5;
+        const bool lead = (threadIdx.x & 31) == 0;
+        for (int tile = blockIdx.x * NWG + gg; tile < ntiles; tile += gridDim.x * NWG) {
+            pair_sync(kBarWritten + gg);
+            if (sm.fail[gg] < 0) break;  // the group gave up
+            const bool fail = tile_fails<VK>(ip, g, vp, *coef, dtf, trace, tile, tiles_x, kstep, chk);
+            if (lead) {
+                sm.fail[gg] = fail;
+                atomicAdd(chk.tiles, 1ull);
+                if (fail) atomicAdd(chk.fallbacks, 1ull);
             }
-        } else if (w.r < chk.samples) {
-            const int q = (int)(tile_hash((uint32_t)tile, (uint32_t)kstep + 977u * w.r) % (uint32_t)width);
-            const float *yq = &outs[q * 8];
-            const float xq = g.lo0 + (float)(x0 + q) * g.h0, yy = g.lo1 + (float)j * g.h1;
-            float dr[2], Jr[4];
-            trace2d<TR_RK3, VK>(vp, *coef, xq, yy, dtf, dr[0], dr[1], Jr);
-            const float ex = fmaxf(fabsf(yq[0] * ip.scale[0] * g.h0 - dr[0]) * g.ih0,
-                                   fabsf(yq[1] * ip.scale[1] * g.h1 - dr[1]) * g.ih1);
-            const float mJ[4] = {1.f + dtf * yq[2] * ip.scale[2], dtf * yq[3] * ip.scale[3],
-                                 dtf * yq[4] * ip.scale[4], 1.f + dtf * yq[5] * ip.scale[5]};
-            float eJ = 0.f;
-            for (int e = 0; e < 4; ++e) eJ = fmaxf(eJ, fabsf(mJ[e] - Jr[e]));
-            if (!(ex <= chk.tol_x) || !(eJ <= chk.tol_J)) atomicOr(&sm.fail[w.g], 1);
+            pair_arrive(kBarChecked + gg);
         }
-        wg_sync(w.g);
-        const bool fail = sm.fail[w.g] != 0;
-        if (fail && i < g.n0) {
-            const float x = g.lo0 + (float)i * g.h0, yy = g.lo1 + (float)j * g.h1;
-            trace2d<TR_RK3, VK>(vp, *coef, x, yy, dtf, d[0], d[1], J);
-        }
-        if (i < g.n0) {
+    } else {
+        Wg w = make_wg(sm);
+        bool aborted = false;
+        const double t = t_dev[0] + (double)kstep * dt;
+        const float phase = (float)(t - floor(t));
+        int prev = -1;
+        auto store = [&](int j, int i, const float (&d)[2], const float (&J)[4]) {
             const int64_t o = (int64_t)j * g.pitch + i;
             trace[o] = d[0];
             trace[g.plane + o] = d[1];
-            trace[2 * g.plane + o] = J[0];
-            trace[3 * g.plane + o] = J[1];
-            trace[4 * g.plane + o] = J[2];
-            trace[5 * g.plane + o] = J[3];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) trace[(2 + e) * g.plane + o] = J[e];
+        };
+        auto finish = [&](int tile) {  // the check's verdict on a tile written earlier
+            pair_sync(kBarChecked + w.g);
+            const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
+            if (sm.fail[w.g] && i < g.n0) {
+                float d[2], J[4];
+                trace2d<TR_RK3, VK>(vp, *coef, g.lo0 + (float)i * g.h0, g.lo1 + (float)j * g.h1, dtf, d[0], d[1], J);
+                store(j, i, d, J);
+            }
+        };
+        for (int tile = blockIdx.x * NWG + w.g; tile < ntiles; tile += gridDim.x * NWG) {
+            const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
+            {
+                const float x = g.lo0 + (float)min(i, g.n0 - 1) * g.h0, y = g.lo1 + (float)j * g.h1;
+                stage_input(sm, w, 2.f * x - 1.f, 2.f * y - 1.f, 2.f * phase - 1.f);
+            }
+            float y[8];
+            if (!run_tile(sm, w, chk.err, y)) { aborted = true; break; }
+            if (i < g.n0) {
+                float d[2], J[4];
+                d[0] = y[0] * ip.scale[0] * g.h0;
+                d[1] = y[1] * ip.scale[1] * g.h1;
+                J[0] = 1.f + dtf * y[2] * ip.scale[2];
+                J[1] = dtf * y[3] * ip.scale[3];
+                J[2] = dtf * y[4] * ip.scale[4];
+                J[3] = 1.f + dtf * y[5] * ip.scale[5];
+                store(j, i, d, J);
+            }
+            if (prev >= 0) finish(prev);
+            pair_arrive(kBarWritten + w.g);
+            prev = tile;
         }
-        if (w.r == 0) {
-            atomicAdd(chk.tiles, 1ull);
-            if (fail) atomicAdd(chk.fallbacks, 1ull);
+        if (prev >= 0) finish(prev);
+        if (aborted) {  // the checking warp waits for the tile that did not come
+            wg_sync(w.g);
+            sm.fail[w.g] = -1;
+            pair_arrive(kBarWritten + w.g);
         }
-        wg_sync(w.g);  // outs, fail and act[g] are reused by the next tile
+        drain(sm, w, aborted);
     }
-    drain(sm, w, aborted);
     block_teardown(sm);
 }
 
@@ -467,7 +498,7 @@ cudaError_t launch_mlp_trace(const InferParams &ip, const Geom &g, const VelPara
     const int ntiles = ((g.n0 + ROWS - 1) / ROWS) * g.n1, sms = sm_count();
     const int blocks = (ntiles + NWG - 1) / NWG;
     auto kern = vp.kind == VK_WAVES2D ? k_mlp_trace<VK_WAVES2D> : k_mlp_trace<VK_FOURIER2D>;
-    kern<<<blocks < sms ? blocks : sms, NT, sizeof(Smem), s>>>(ip, g, vp, coef, t_dev, kstep, dt, trace, chk);
+    kern<<<blocks < sms ? blocks : sms, NTT, sizeof(Smem), s>>>(ip, g, vp, coef, t_dev, kstep, dt, trace, chk);
     return cudaGetLastError();
 }
 
