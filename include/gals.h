@@ -160,8 +160,11 @@ gals_status gals_set_state(gals_grid *grid, const float *const *fields, int nfie
  * (outflow or tangential boundaries need no data, Sec. 4.1).  nsteps > 1 is replayed
  * from cached CUDA graphs of at most 256 steps each (of one launch per step, or of one
  * persistent launch, see gals_set_time_loop); each graph reads the grid clock on the
- * device and advances it, so longer calls replay the same graph.  In 2D the graph splits each step into up to 4 bands of whole tile
- * rows, at least 2 tiles and the velocity's reach plus 4 rows high; a band of step s
+ * device and advances it, so longer calls replay the same graph.  In the FULL layout only a
+ * run's first step reads the stored mixed derivatives and only its last one writes them;
+ * the steps between rebuild them from the gradients, the same values (in 3D where the feet
+ * stay near their node; else every step writes them).  In 2D the graph splits each step
+ * into up to 4 bands of whole tile rows, at least 2 tiles and the velocity's reach plus 4 rows high; a band of step s
  * depends only on itself and its two neighbouring bands at step s - 1, so the next step's
  * bands start while the current one drains (same results bit for bit).  A run of 8 or more
  * steps on a 2D grid of at most 12288 nodes (rows of at most 512) is one launch of a
@@ -182,8 +185,9 @@ gals_status gals_step(gals_grid *grid, const gals_velocity *vel, double dt, int 
  *               around it have finished step s - 1, so no step waits for the last tiles of
  *               the previous one to drain; elsewhere one launch per step.  On a GB300 it
  *               runs slower than LAUNCHES on the 4096^2 single vortex (0.148 ms per step
- *               against 0.128 ms for the banded graph): the per-tile flag fence and acquire
- *               cost more than the drained tails it saves.
+ *               against 0.107 ms for the banded graph): it writes the mixed derivatives in
+ *               every step, and the per-tile flag fence and acquire cost more than the
+ *               drained tails it saves.
  * Both give the same results bit for bit. */
 enum { GALS_LOOP_LAUNCHES = 0, GALS_LOOP_PERSISTENT = 1 };
 
