@@ -291,12 +291,13 @@ __device__ __forceinline__ void pair_arrive(int id)
 constexpr int kBarWritten = 1 + NWG, kBarChecked = 1 + 2 * NWG;
 constexpr int NTT = NT + 32 * NWG;  // threads per block of the trace kernel
 
-// Whether one of the tile's sampled nodes is off the exact RK3 trace: warp-wide, the
-// network's values read back from the trace planes.
-template <int VK>
+// Whether one of the tile's sampled nodes (first, first + stride, ...; for a cheap field all of
+// them, one per lane) is off the exact RK3 trace: warp-wide; value(q, e): the network's values
+// of the tile's node q, delta and J.
+template <int VK, class V>
 __device__ __forceinline__ bool tile_fails(const InferParams &ip, const Geom &g, const VelParams &vp,
-                                           const StageCoef &coef, float dtf, const float *trace, int tile, int tiles_x,
-                                           int kstep, const Check &chk)
+                                           const StageCoef &coef, float dtf, V value, int tile, int tiles_x,
+                                           int kstep, const Check &chk, int first, int stride)
 {
     const int lane = threadIdx.x & 31;
     const int j = tile / tiles_x, x0 = (tile % tiles_x) * ROWS, width = min(ROWS, g.n0 - x0);
@@ -304,13 +305,12 @@ __device__ __forceinline__ bool tile_fails(const InferParams &ip, const Geom &g,
     bool bad = false;
     // a costly field: each node's trace by the whole warp (modes split over the lanes)
     constexpr bool WARP = VK == VK_WAVES2D;
-    for (int jj = WARP ? 0 : lane; jj < chk.samples; jj += WARP ? 1 : 32) {
+    for (int jj = WARP ? first : lane; jj < chk.samples; jj += WARP ? stride : 32) {
         const int q = (int)(tile_hash((uint32_t)tile, (uint32_t)kstep + 977u * jj) % (uint32_t)width);
         const float xq = g.lo0 + (float)(x0 + q) * g.h0;
         float dr[2], Jr[4], m[6];
-        const int64_t o = (int64_t)j * g.pitch + x0 + q;
 #pragma unroll
-        for (int e = 0; e < 6; ++e) m[e] = trace[e * g.plane + o];
+        for (int e = 0; e < 6; ++e) m[e] = value(q, e);
         if (WARP) trace2d_waves_warp(vp, coef, xq, yy, dtf, dr[0], dr[1], Jr);
         else trace2d<TR_RK3, VK>(vp, coef, xq, yy, dtf, dr[0], dr[1], Jr);
         const float ex = fmaxf(fabsf(m[0] - dr[0]) * g.ih0, fabsf(m[1] - dr[1]) * g.ih1);
@@ -329,8 +329,15 @@ __device__ __forceinline__ bool tile_fails(const InferParams &ip, const Geom &g,
 // runs the next one, and the group recomputes a tile that failed one tile later.  2048^2,
 // 16 modes, a whole step: 794 -> 733 us with 4 nodes, 809 -> 766 with 128 nodes a tile (four
 // rounds of the warp), 876 -> 842 where every tile fails; 500^2 70.5 -> 68.
+//
+// A costly field keeps the check in the group, a sample per warp with its modes over the
+// lanes: one warp alone falls behind the network.  2048^2, us per step in the group / aside:
+// 256 waves, 4 nodes 926 / 811, 16 nodes 1397 / 2259, every tile failing 3443 / 3996; 1024
+// waves, 4 nodes 1382 / 2262.
+template <int VK> constexpr bool aside() { return VK != VK_WAVES2D; }
+
 template <int VK>
-__global__ void __launch_bounds__(NTT, 1)
+__global__ void __launch_bounds__(aside<VK>() ? NTT : NT, 1)
 k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ coef,
             const double *__restrict__ t_dev, int kstep, double dt, float *trace, Check chk)
 {
@@ -340,13 +347,15 @@ k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ 
     const float dtf = (float)dt;
     const int tiles_x = (g.n0 + ROWS - 1) / ROWS;
     const int ntiles = tiles_x * g.n1;
-    if (threadIdx.x >= NT) {
+    if (aside<VK>() && threadIdx.x >= NT) {
         const int gg = (threadIdx.x - NT) >> 5;
         const bool lead = (threadIdx.x & 31) == 0;
         for (int tile = blockIdx.x * NWG + gg; tile < ntiles; tile += gridDim.x * NWG) {
             pair_sync(kBarWritten + gg);
             if (sm.fail[gg] < 0) break;  // the group gave up
-            const bool fail = tile_fails<VK>(ip, g, vp, *coef, dtf, trace, tile, tiles_x, kstep, chk);
+            const float *at = trace + (int64_t)(tile / tiles_x) * g.pitch + (tile % tiles_x) * ROWS;
+            auto value = [&](int q, int e) { return at[e * g.plane + q]; };
+            const bool fail = tile_fails<VK>(ip, g, vp, *coef, dtf, value, tile, tiles_x, kstep, chk, 0, 1);
             if (lead) {
                 sm.fail[gg] = fail;
                 atomicAdd(chk.tiles, 1ull);
@@ -367,14 +376,16 @@ k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ 
 #pragma unroll
             for (int e = 0; e < 4; ++e) trace[(2 + e) * g.plane + o] = J[e];
         };
+        auto exact = [&](int tile) {
+            const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
+            if (i >= g.n0) return;
+            float d[2], J[4];
+            trace2d<TR_RK3, VK>(vp, *coef, g.lo0 + (float)i * g.h0, g.lo1 + (float)j * g.h1, dtf, d[0], d[1], J);
+            store(j, i, d, J);
+        };
         auto finish = [&](int tile) {  // the check's verdict on a tile written earlier
             pair_sync(kBarChecked + w.g);
-            const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
-            if (sm.fail[w.g] && i < g.n0) {
-                float d[2], J[4];
-                trace2d<TR_RK3, VK>(vp, *coef, g.lo0 + (float)i * g.h0, g.lo1 + (float)j * g.h1, dtf, d[0], d[1], J);
-                store(j, i, d, J);
-            }
+            if (sm.fail[w.g]) exact(tile);
         };
         for (int tile = blockIdx.x * NWG + w.g; tile < ntiles; tile += gridDim.x * NWG) {
             const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
@@ -384,22 +395,36 @@ k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ 
             }
             float y[8];
             if (!run_tile(sm, w, chk.err, y)) { aborted = true; break; }
-            if (i < g.n0) {
-                float d[2], J[4];
-                d[0] = y[0] * ip.scale[0] * g.h0;
-                d[1] = y[1] * ip.scale[1] * g.h1;
-                J[0] = 1.f + dtf * y[2] * ip.scale[2];
-                J[1] = dtf * y[3] * ip.scale[3];
-                J[2] = dtf * y[4] * ip.scale[4];
-                J[3] = 1.f + dtf * y[5] * ip.scale[5];
-                store(j, i, d, J);
+            float d[2], J[4];
+            d[0] = y[0] * ip.scale[0] * g.h0;
+            d[1] = y[1] * ip.scale[1] * g.h1;
+            J[0] = 1.f + dtf * y[2] * ip.scale[2];
+            J[1] = dtf * y[3] * ip.scale[3];
+            J[2] = dtf * y[4] * ip.scale[4];
+            J[3] = 1.f + dtf * y[5] * ip.scale[5];
+            if (!aside<VK>()) {
+                float *outs = reinterpret_cast<float *>(sm.act[w.g]);  // free after the products
+#pragma unroll
+                for (int e = 0; e < 6; ++e) outs[w.r * 8 + e] = e < 2 ? d[e] : J[e - 2];
+                wg_sync(w.g);
+                auto value = [&](int q, int e) { return outs[q * 8 + e]; };
+                const bool fail = wg_sync_or(w.g, tile_fails<VK>(ip, g, vp, *coef, dtf, value, tile, tiles_x, kstep,
+                                                                 chk, w.r >> 5, GT / 32));
+                if (fail) exact(tile);
+                else if (i < g.n0) store(j, i, d, J);
+                if (w.r == 0) {
+                    atomicAdd(chk.tiles, 1ull);
+                    if (fail) atomicAdd(chk.fallbacks, 1ull);
+                }
+                continue;
             }
+            if (i < g.n0) store(j, i, d, J);
             if (prev >= 0) finish(prev);
             pair_arrive(kBarWritten + w.g);
             prev = tile;
         }
         if (prev >= 0) finish(prev);
-        if (aborted) {  // the checking warp waits for the tile that did not come
+        if (aside<VK>() && aborted) {  // the checking warp waits for the tile that did not come
             wg_sync(w.g);
             sm.fail[w.g] = -1;
             pair_arrive(kBarWritten + w.g);
@@ -498,7 +523,8 @@ cudaError_t launch_mlp_trace(const InferParams &ip, const Geom &g, const VelPara
     const int ntiles = ((g.n0 + ROWS - 1) / ROWS) * g.n1, sms = sm_count();
     const int blocks = (ntiles + NWG - 1) / NWG;
     auto kern = vp.kind == VK_WAVES2D ? k_mlp_trace<VK_WAVES2D> : k_mlp_trace<VK_FOURIER2D>;
-    kern<<<blocks < sms ? blocks : sms, NTT, sizeof(Smem), s>>>(ip, g, vp, coef, t_dev, kstep, dt, trace, chk);
+    const int threads = vp.kind == VK_WAVES2D ? NT : NTT;  // aside()
+    kern<<<blocks < sms ? blocks : sms, threads, sizeof(Smem), s>>>(ip, g, vp, coef, t_dev, kstep, dt, trace, chk);
     return cudaGetLastError();
 }
 
