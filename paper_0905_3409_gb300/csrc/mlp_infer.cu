@@ -376,16 +376,14 @@ k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ 
 #pragma unroll
             for (int e = 0; e < 4; ++e) trace[(2 + e) * g.plane + o] = J[e];
         };
-        auto exact = [&](int tile) {
-            const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
-            if (i >= g.n0) return;
-            float d[2], J[4];
-            trace2d<TR_RK3, VK>(vp, *coef, g.lo0 + (float)i * g.h0, g.lo1 + (float)j * g.h1, dtf, d[0], d[1], J);
-            store(j, i, d, J);
-        };
         auto finish = [&](int tile) {  // the check's verdict on a tile written earlier
             pair_sync(kBarChecked + w.g);
-            if (sm.fail[w.g]) exact(tile);
+            const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
+            if (sm.fail[w.g] && i < g.n0) {
+                float d[2], J[4];
+                trace2d<TR_RK3, VK>(vp, *coef, g.lo0 + (float)i * g.h0, g.lo1 + (float)j * g.h1, dtf, d[0], d[1], J);
+                store(j, i, d, J);
+            }
         };
         for (int tile = blockIdx.x * NWG + w.g; tile < ntiles; tile += gridDim.x * NWG) {
             const int j = tile / tiles_x, i = (tile % tiles_x) * ROWS + w.r;
@@ -410,8 +408,9 @@ k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ 
                 auto value = [&](int q, int e) { return outs[q * 8 + e]; };
                 const bool fail = wg_sync_or(w.g, tile_fails<VK>(ip, g, vp, *coef, dtf, value, tile, tiles_x, kstep,
                                                                  chk, w.r >> 5, GT / 32));
-                if (fail) exact(tile);
-                else if (i < g.n0) store(j, i, d, J);
+                if (fail && i < g.n0)
+                    trace2d<TR_RK3, VK>(vp, *coef, g.lo0 + (float)i * g.h0, g.lo1 + (float)j * g.h1, dtf, d[0], d[1], J);
+                if (i < g.n0) store(j, i, d, J);
                 if (w.r == 0) {
                     atomicAdd(chk.tiles, 1ull);
                     if (fail) atomicAdd(chk.fallbacks, 1ull);
@@ -423,7 +422,7 @@ k_mlp_trace(InferParams ip, Geom g, VelParams vp, const StageCoef *__restrict__ 
             pair_arrive(kBarWritten + w.g);
             prev = tile;
         }
-        if (prev >= 0) finish(prev);
+        if (aside<VK>() && prev >= 0) finish(prev);
         if (aside<VK>() && aborted) {  // the checking warp waits for the tile that did not come
             wg_sync(w.g);
             sm.fail[w.g] = -1;
