@@ -44,8 +44,12 @@ constexpr int64_t kShortTileBlocks = GALS_SHORT_BLOCKS;
 // set-up being nothing beside them: short tiles on any grid, because a step's few waves of
 // tall ones leave the last one part empty (2048^2: 2516 tiles on 760 places).  256 waves: 2048^2 1.60 -> 1.49 ms
 // per step, 1000^2 476 -> 371 us, 700^2 with 512 707 -> 377; the floor of the sines and
-// cosines is 1.28 ms at 2048^2.  With 16 and 32 waves both shapes take the same time.
+// cosines is 1.28 ms at 2048^2.  With 16 and 32 waves both shapes take the same time.  Grids
+// of more rows than a launch of short tiles holds (65535 tiles along y) keep the tall ones,
+// whose number the grid's size limit is made for; the rule looks at the whole grid, so that
+// every band of a step decides alike.
 constexpr int kShortWaves = 64;
+constexpr int kMaxShortRows = 65535 * TYS;
 
 template <int WC> constexpr bool overlapped() { return OVX && WC; }
 template <int WC> constexpr int tile_stride() { return overlapped<WC>() ? TX - 2 : TX; }
@@ -231,7 +235,8 @@ cudaError_t launch_ty(const StepLaunch &a, cudaStream_t s)
 template <int TR, int VK, int CR, int WC>
 cudaError_t launch_t(const StepLaunch &a, cudaStream_t s)
 {
-    const bool is_short = short_tiles(a.geom) || (VK == VK_WAVES2D && a.vp.nwaves >= kShortWaves);
+    const bool is_short = short_tiles(a.geom) ||
+                          (VK == VK_WAVES2D && a.vp.nwaves >= kShortWaves && a.geom.n1 <= kMaxShortRows);
     return is_short ? launch_ty<TYS, TR, VK, CR, WC>(a, s) : launch_ty<TY, TR, VK, CR, WC>(a, s);
 }
 
