@@ -169,13 +169,9 @@ cudaError_t launch_t(const BatchLaunch &a, cudaStream_t s)
 {
     constexpr int NP = CR == CROSS_PLANE ? 4 : 3;
     auto kern = k_batch2d<TY, VK, CR, WC>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             Geo<TY>::bytes(NP));
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice ready;
+    cudaError_t e = ready.once([&] { return allow_dynamic_smem(kern, Geo<TY>::bytes(NP)); });
+    if (e != cudaSuccess) return e;
     const int grid = a.grid > 0 ? a.grid : a.nitems;
     kern<<<grid, TX, Geo<TY>::bytes(NP), s>>>(a.in, a.out, a.probs, a.vps, a.coef, a.maps[NP - 3],
                                               a.items, a.nitems, a.err);
@@ -187,15 +183,15 @@ cudaError_t launch_run_t(const BatchRunLaunch &a, cudaStream_t s)
 {
     constexpr int NP = CR == CROSS_PLANE ? 4 : 3;
     auto kern = k_batch2d_run<TY, VK, CR, WC>;
-    static int blocks_per_sm = 0;  // per instantiation
-    if (blocks_per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Geo<TY>::bytes(NP));
-        if (e != cudaSuccess) return e;
-        int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, TX, Geo<TY>::bytes(NP));
-        if (e != cudaSuccess) return e;
-        blocks_per_sm = nb > 0 ? nb : 1;
-    }
+    static PerDevice fit;  // per instantiation
+    int blocks_per_sm = 0;
+    cudaError_t e = fit.get(&blocks_per_sm, [&](int *nb) {
+        cudaError_t a = allow_dynamic_smem(kern, Geo<TY>::bytes(NP));
+        if (a == cudaSuccess) a = cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, kern, TX, Geo<TY>::bytes(NP));
+        if (*nb < 1) *nb = 1;
+        return a;
+    });
+    if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

@@ -368,10 +368,13 @@ cudaError_t issue_steps(gals_grid *g, const VelParams &vp, int trace, double dt,
     return launch_advance_time(g->t_dev, nsteps, dt, g->stream, chain);
 }
 
-// A run on a small 2D grid: coefficients, one cluster launch, clock.
+// A run on a small 2D grid: coefficients, one cluster launch, clock.  done: false if the device
+// cannot place the cluster (the coefficients, which any other way computes again, are all that
+// is queued then).
 cudaError_t issue_small(gals_grid *g, const VelParams &vp, int trace, double dt, int nsteps, bool first_explicit,
-                        int64_t &launches)
+                        int64_t &launches, bool *done)
 {
+    *done = false;
     launches = (vp.kind == VK_WAVES2D ? 2 : 1) + 2;
     cudaError_t ce = launch_coef_table(g->coef, vp, g->t_dev, dt, nsteps, g->stream);
     if (ce != cudaSuccess) return ce;
@@ -388,7 +391,7 @@ cudaError_t issue_small(gals_grid *g, const VelParams &vp, int trace, double dt,
     r.planes = a.cross_in == CROSS_PLANE;
     r.write_cross = a.write_cross;
     r.nsteps = nsteps;
-    if ((ce = launch_step2d_small(r, g->stream)) != cudaSuccess) return ce;
+    if ((ce = launch_step2d_small(r, g->stream, done)) != cudaSuccess || !*done) return ce;
     return launch_advance_time(g->t_dev, nsteps, dt, g->stream);
 }
 
@@ -759,12 +762,15 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
         }
         if (use_small(g, v->trace, cs)) {
             int64_t nl = 0;
-            if ((ce = issue_small(g, vp, v->trace, dt, cs, fe_c, nl)) != cudaSuccess) {
+            bool small = false;
+            if ((ce = issue_small(g, vp, v->trace, dt, cs, fe_c, nl, &small)) != cudaSuccess) {
                 what = "small-grid launch";
                 return ce;
             }
-            total += nl;
-            return cudaSuccess;
+            if (small) {
+                total += nl;
+                return cudaSuccess;
+            }
         }
         GraphEntry *hit = nullptr;
         for (auto &ge : g->graphs)

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "gals_device.cuh"
+#include "per_device.h"
 
 namespace gals {
 
@@ -96,7 +97,8 @@ struct SmallLaunch {
     int nsteps;
 };
 bool small2d_fits(const Geom &g);
-cudaError_t launch_step2d_small(const SmallLaunch &a, cudaStream_t s);
+// done: false if the current device cannot place the cluster (nothing is queued then)
+cudaError_t launch_step2d_small(const SmallLaunch &a, cudaStream_t s, bool *done);
 
 // Granularity of StepLaunch bands: the 2D tile height, the 3D tile depth.
 int band_unit(int dim);

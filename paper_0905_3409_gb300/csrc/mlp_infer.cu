@@ -474,12 +474,6 @@ int sm_count()
     return sms > 0 ? sms : 1;
 }
 
-template <class K>
-cudaError_t set_smem(K fn)
-{
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
-}
-
 static_assert(sizeof(Smem) <= 227 * 1024, "shared memory budget");
 static_assert(W_TOTAL * 2 % 16 == 0, "weights are copied in 16-byte chunks");
 static_assert(W2_OFF * 2 % 16 == 0 && W5_OFF * 2 % 16 == 0 && WB_OFF * 2 % 16 == 0 &&
@@ -496,12 +490,9 @@ cudaError_t pack_infer(const float *params, InferParams &ip, cudaStream_t s)
 
 cudaError_t infer_points(const InferParams &ip, const float *Xn, float *Y, int n, int *err, cudaStream_t s)
 {
-    static bool set = false;
-    if (!set) {
-        cudaError_t e = set_smem(k_infer_points);
-        if (e != cudaSuccess) return e;
-        set = true;
-    }
+    static PerDevice ready;
+    cudaError_t e = ready.once([] { return allow_dynamic_smem(k_infer_points, (int)sizeof(Smem)); });
+    if (e != cudaSuccess) return e;
     const int tiles = (n + ROWS - 1) / ROWS, sms = sm_count();
     const int blocks = (tiles + NWG - 1) / NWG;
     k_infer_points<<<blocks < sms ? blocks : sms, NT, sizeof(Smem), s>>>(ip, Xn, Y, n, err);
@@ -512,13 +503,12 @@ cudaError_t launch_mlp_trace(const InferParams &ip, const Geom &g, const VelPara
                              const StageCoef *coef, const double *t_dev, int kstep, double dt,
                              float *trace, const Check &chk, cudaStream_t s)
 {
-    static bool set = false;
-    if (!set) {
-        cudaError_t e = set_smem(k_mlp_trace<VK_FOURIER2D>);
-        if (e == cudaSuccess) e = set_smem(k_mlp_trace<VK_WAVES2D>);
-        if (e != cudaSuccess) return e;
-        set = true;
-    }
+    static PerDevice ready;
+    cudaError_t e = ready.once([] {
+        const cudaError_t a = allow_dynamic_smem(k_mlp_trace<VK_FOURIER2D>, (int)sizeof(Smem));
+        return a != cudaSuccess ? a : allow_dynamic_smem(k_mlp_trace<VK_WAVES2D>, (int)sizeof(Smem));
+    });
+    if (e != cudaSuccess) return e;
     const int ntiles = ((g.n0 + ROWS - 1) / ROWS) * g.n1, sms = sm_count();
     const int blocks = (ntiles + NWG - 1) / NWG;
     auto kern = vp.kind == VK_WAVES2D ? k_mlp_trace<VK_WAVES2D> : k_mlp_trace<VK_FOURIER2D>;

@@ -411,14 +411,9 @@ cudaError_t pack_train(const float *params, uint16_t *wt, cudaStream_t s)
 cudaError_t launch_train_tiles(const float *params, const uint16_t *wt, const float *X, const float *T, int n,
                                float *Zs, float *part, double *loss, int *err, cudaStream_t s)
 {
-    static bool set = false;
-    cudaError_t e;
-    if (!set) {
-        if ((e = cudaFuncSetAttribute(k_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem))) !=
-            cudaSuccess)
-            return e;
-        set = true;
-    }
+    static PerDevice ready;
+    cudaError_t e = ready.once([] { return allow_dynamic_smem(k_train_tile, (int)sizeof(TrainSmem)); });
+    if (e != cudaSuccess) return e;
     if (loss && (e = cudaMemsetAsync(loss, 0, sizeof(double), s)) != cudaSuccess) return e;
     const int nsplit = train_splits(n), chunk = (n + nsplit - 1) / nsplit;
     k_train_tile<<<nsplit, TT, sizeof(TrainSmem), s>>>(params, wt, X, T, n, chunk, reinterpret_cast<float4 *>(Zs), part,

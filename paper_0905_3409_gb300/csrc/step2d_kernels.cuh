@@ -211,14 +211,12 @@ cudaError_t launch_ty(const StepLaunch &a, cudaStream_t s)
 {
     constexpr int NP = CR == CROSS_PLANE ? 4 : 3;
     constexpr int bytes = Geo<TYT, HYT, TWS>::bytes(NP);
-    static bool attr_set = false;  // one attribute call per instantiation (not a stream op)
-    if (!attr_set) {
-        cudaError_t e;
-        if constexpr (!walked<TYT, VK, CR, WC>()) e = cudaFuncSetAttribute(k_step2d<TYT, TR, VK, CR, WC>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        else e = cudaFuncSetAttribute(k_walk2d<TYT, TR, VK, CR>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice ready;  // one attribute call per instantiation and device (not a stream op)
+    cudaError_t e = ready.once([] {
+        if constexpr (!walked<TYT, VK, CR, WC>()) return allow_dynamic_smem(k_step2d<TYT, TR, VK, CR, WC>, bytes);
+        else return allow_dynamic_smem(k_walk2d<TYT, TR, VK, CR>, bytes);
+    });
+    if (e != cudaSuccess) return e;
     // rows of the band (all by default)
     const int row0 = a.band_lo, row1 = a.band_hi > 0 ? a.band_hi : a.geom.n1;
     if (row1 <= row0) return cudaSuccess;
@@ -262,15 +260,15 @@ template <int TR, int VK>
 cudaError_t launch_run_t(const RunLaunch &a, cudaStream_t s)
 {
     auto kern = k_step2d_run<TR, VK>;
-    static int blocks_per_sm = 0;  // per instantiation
-    if (blocks_per_sm == 0) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, GT::bytes(4));
-        if (e != cudaSuccess) return e;
-        int nb = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, TX, GT::bytes(4));
-        if (e != cudaSuccess) return e;
-        blocks_per_sm = nb > 0 ? nb : 1;
-    }
+    static PerDevice fit;  // per instantiation
+    int blocks_per_sm = 0;
+    cudaError_t e = fit.get(&blocks_per_sm, [&](int *nb) {
+        cudaError_t a = allow_dynamic_smem(kern, GT::bytes(4));
+        if (a == cudaSuccess) a = cudaOccupancyMaxActiveBlocksPerMultiprocessor(nb, kern, TX, GT::bytes(4));
+        if (*nb < 1) *nb = 1;
+        return a;
+    });
+    if (e != cudaSuccess) return e;
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

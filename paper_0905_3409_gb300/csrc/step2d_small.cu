@@ -226,11 +226,10 @@ int rows_per_block(int n1, int cluster) { return (n1 + 2 * cluster - 1) / (2 * c
 size_t small_bytes(const Geom &g, int R) { return sizeof(float4) * 2 * (size_t)R * g.n0; }
 
 template <int TR, int VK, int CR>
-cudaError_t launch_t(const SmallLaunch &a, cudaStream_t s)
+cudaError_t launch_t(const SmallLaunch &a, cudaStream_t s, bool *done)
 {
     auto kern = k_step2d_small<TR, VK, CR>;
-    static int cluster = 0;  // per instantiation: 16 blocks where the device can place them, else 8
-    cudaError_t e;
+    static PerDevice fit;  // per instantiation
     cudaLaunchConfig_t cfg{};
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeClusterDimension;
@@ -238,21 +237,25 @@ cudaError_t launch_t(const SmallLaunch &a, cudaStream_t s)
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     cfg.stream = s;
-    if (cluster == 0) {
-        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmallMaxBytes)) != cudaSuccess ||
-            (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-            return e;
-        int nc = 0;
-        at.val.clusterDim.x = kSmallCluster;
-        cfg.gridDim = dim3(kSmallCluster);
+    // 16 blocks where the device can place them, else 8, else (0) no cluster at all
+    int cluster = 0;
+    cudaError_t e = fit.get(&cluster, [&](int *out) {
+        const bool smem = allow_dynamic_smem(kern, kSmallMaxBytes) == cudaSuccess;
+        const bool large = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
         cfg.blockDim = dim3(kSmallThreads);
         cfg.dynamicSmemBytes = kSmallMaxBytes;
-        if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) != cudaSuccess) {
-            cudaGetLastError();
-            nc = 0;
+        *out = large ? kSmallCluster : 8;
+        for (int nc = 0; smem && *out >= 8; *out /= 2) {
+            at.val.clusterDim.x = *out;
+            cfg.gridDim = dim3(*out);
+            if (cudaOccupancyMaxActiveClusters(&nc, kern, &cfg) == cudaSuccess && nc >= 1) break;
         }
-        cluster = nc >= 1 ? kSmallCluster : 8;
-    }
+        cudaGetLastError();  // of what this device does not have
+        if (!smem || *out < 8) *out = 0;
+        return cudaSuccess;
+    });
+    if (e != cudaSuccess || cluster == 0) return e;
+    *done = true;
     const int R = rows_per_block(a.geom.n1, cluster);
     const int pairs = (R / 2) * a.geom.n0;
     at.val.clusterDim.x = cluster;
@@ -264,16 +267,16 @@ cudaError_t launch_t(const SmallLaunch &a, cudaStream_t s)
 }
 
 template <int TR, int VK>
-cudaError_t launch_cr(const SmallLaunch &a, cudaStream_t s)
+cudaError_t launch_cr(const SmallLaunch &a, cudaStream_t s, bool *done)
 {
-    return a.cell ? launch_t<TR, VK, CROSS_CELL>(a, s) : launch_t<TR, VK, CROSS_RECON>(a, s);
+    return a.cell ? launch_t<TR, VK, CROSS_CELL>(a, s, done) : launch_t<TR, VK, CROSS_RECON>(a, s, done);
 }
 
 template <int VK>
-cudaError_t launch_tr(const SmallLaunch &a, cudaStream_t s)
+cudaError_t launch_tr(const SmallLaunch &a, cudaStream_t s, bool *done)
 {
-    if (a.trace == TR_HEUN) return launch_cr<TR_HEUN, VK>(a, s);
-    return a.trace == TR_EULER ? launch_cr<TR_EULER, VK>(a, s) : launch_cr<TR_RK3, VK>(a, s);
+    if (a.trace == TR_HEUN) return launch_cr<TR_HEUN, VK>(a, s, done);
+    return a.trace == TR_EULER ? launch_cr<TR_EULER, VK>(a, s, done) : launch_cr<TR_RK3, VK>(a, s, done);
 }
 
 }  // namespace
@@ -285,15 +288,16 @@ bool small2d_fits(const Geom &g)
            small_bytes(g, rows_per_block(g.n1, 8)) <= (size_t)kSmallMaxBytes;
 }
 
-cudaError_t launch_step2d_small(const SmallLaunch &a, cudaStream_t s)
+cudaError_t launch_step2d_small(const SmallLaunch &a, cudaStream_t s, bool *done)
 {
+    *done = false;
     switch (a.vp.kind) {
-    case VK_CONST: return launch_tr<VK_CONST>(a, s);
-    case VK_ROTATION: return launch_tr<VK_ROTATION>(a, s);
-    case VK_VORTEX2D: return launch_tr<VK_VORTEX2D>(a, s);
-    case VK_PSEUDO1D: return launch_tr<VK_PSEUDO1D>(a, s);
-    case VK_FOURIER2D: return launch_tr<VK_FOURIER2D>(a, s);
-    case VK_WAVES2D: return launch_tr<VK_WAVES2D>(a, s);
+    case VK_CONST: return launch_tr<VK_CONST>(a, s, done);
+    case VK_ROTATION: return launch_tr<VK_ROTATION>(a, s, done);
+    case VK_VORTEX2D: return launch_tr<VK_VORTEX2D>(a, s, done);
+    case VK_PSEUDO1D: return launch_tr<VK_PSEUDO1D>(a, s, done);
+    case VK_FOURIER2D: return launch_tr<VK_FOURIER2D>(a, s, done);
+    case VK_WAVES2D: return launch_tr<VK_WAVES2D>(a, s, done);
     default: return cudaErrorInvalidValue;
     }
 }

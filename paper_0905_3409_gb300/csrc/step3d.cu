@@ -429,13 +429,9 @@ template <int TR, int VK, int CR>
 cudaError_t launch_t(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
     using T = Tile3<CR>;
-    static bool attr_set = false;
-    if (!attr_set) {
-        cudaError_t e = cudaFuncSetAttribute(k_step3d<TR, VK, CR>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
-        if (e != cudaSuccess) return e;
-        attr_set = true;
-    }
+    static PerDevice ready;
+    cudaError_t e = ready.once([] { return allow_dynamic_smem(k_step3d<TR, VK, CR>, T::SMEM); });
+    if (e != cudaSuccess) return e;
     dim3 block(TX, TY);
     dim3 grid((a.geom.n0 + TX - 1) / TX, (a.geom.n1 + TY - 1) / TY, (z1 - z0 + TZ - 1) / TZ);
     const CUtensorMap &map = *a.tmap[0][CR == CROSS_PLANE];
