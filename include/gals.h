@@ -169,7 +169,8 @@ gals_status gals_set_state(gals_grid *grid, const float *const *fields, int nfie
  * bands start while the current one drains (same results bit for bit).  A run of 8 or more
  * steps on a 2D grid of at most 12288 nodes (rows of at most 512) is one launch of a
  * thread-block cluster that keeps the state in shared memory (bit for bit too).
- * Asynchronous on the grid stream.
+ * Asynchronous on the grid stream.  nsteps > 1 is refused (GALS_ERR_CUDA) while the
+ * grid's stream is being captured by its owner.
  * Errors: GALS_ERR_ARG (dt <= 0 or non-finite, nsteps < 0, bad velocity descriptor),
  * GALS_ERR_STATE (no state loaded), GALS_ERR_UNSUPPORTED (velocity kind not available in
  * this dimension), GALS_ERR_CUDA (launch failure). */

@@ -761,6 +761,15 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
             return cudaSuccess;
         }
         if (use_small(g, v->trace, cs)) {
+            // refused on a stream under capture, as the capture of a run's graph is: recorded,
+            // the run would move the host's clock and buffers without having taken place
+            cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+            ce = cudaStreamIsCapturing(g->stream, &capturing);
+            if (ce == cudaSuccess && capturing != cudaStreamCaptureStatusNone) ce = cudaErrorIllegalState;
+            if (ce != cudaSuccess) {
+                what = "small-grid run";
+                return ce;
+            }
             int64_t nl = 0;
             bool small = false;
             if ((ce = issue_small(g, vp, v->trace, dt, cs, fe_c, nl, &small)) != cudaSuccess) {
