@@ -843,19 +843,14 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
     return GALS_OK;
 }
 
-// After a stream synchronisation: report (and clear) a kernel-side error word.
-// Wait for the grid's stream and report the error word; copied: queued work stores it in
-// err_host already.
+// Wait for the grid's stream and report (and clear) the error word; copied: queued work
+// stores it in err_host already.
 static gals_status wait_and_check(gals_grid *g, const char *what, bool copied = false)
 {
-    cudaError_t e = cudaSuccess;
-    if (!copied)
-        e = cudaMemcpyAsync(g->err_host, g->err_dev, sizeof(int), cudaMemcpyDeviceToHost, g->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(g->stream);
+    int code = 0;
+    const cudaError_t e = fetch_error_word(g->err_dev, g->err_host, g->stream, copied, &code);
     if (e != cudaSuccess) return cuda_fail(g, e, what);
-    const int code = *(volatile int *)g->err_host;
     if (code == 0) return GALS_OK;
-    cudaMemset(g->err_dev, 0, sizeof(int));
     if ((code & 0xff) == kErrBounds)
         return fail(g, GALS_ERR_CUDA, "checked build: an index left its buffer (source line %d)",
                     code >> 8);

@@ -242,18 +242,14 @@ cudaError_t issue(gals_batch *b, int kind, int nsteps)
     return launch_batch_advance(b->t_dev, b->probs_dev, b->count, nsteps, b->stream);
 }
 
-// Wait for the batch's stream and report the error word; copied: queued work stores it in
-// err_host already.
+// Wait for the batch's stream and report (and clear) the error word; copied: queued work
+// stores it in err_host already.
 gals_status wait_and_check(gals_batch *b, const char *what, bool copied = false)
 {
-    cudaError_t e = cudaSuccess;
-    if (!copied)
-        e = cudaMemcpyAsync(b->err_host, b->err_dev, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+    int code = 0;
+    const cudaError_t e = fetch_error_word(b->err_dev, b->err_host, b->stream, copied, &code);
     if (e != cudaSuccess) return bcuda(b, e, what);
-    const int code = *(volatile int *)b->err_host;
     if (code == 0) return GALS_OK;
-    cudaMemset(b->err_dev, 0, sizeof(int));
     if ((code & 0xff) == kErrBounds)
         return bfail(b, GALS_ERR_CUDA, "checked build: an index left its buffer (source line %d)",
                      code >> 8);

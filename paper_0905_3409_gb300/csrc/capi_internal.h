@@ -22,6 +22,20 @@ struct NvtxRange {
 
 namespace gals {
 
+// Wait for stream s, which a handle's work is ordered on, and fetch the handle's error word into
+// *code (host: its page-locked copy; copied: queued work stores it there already).  A set
+// word is cleared on the same stream: on another one the clear could come after the next
+// read, which would report the error twice, or over the error of newer work.
+inline cudaError_t fetch_error_word(int *dev, int *host, cudaStream_t s, bool copied, int *code)
+{
+    cudaError_t e = cudaSuccess;
+    if (!copied) e = cudaMemcpyAsync(host, dev, sizeof(int), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess) return e;
+    *code = *(volatile int *)host;
+    return *code == 0 ? cudaSuccess : cudaMemsetAsync(dev, 0, sizeof(int), s);
+}
+
 // Validate a velocity descriptor for a grid of dimension `dim` and fill the kernels'
 // parameters; on error writes a message to msg and returns the status.
 gals_status velparams_from(int dim, const gals_velocity *v, VelParams &vp, char *msg, size_t len);
