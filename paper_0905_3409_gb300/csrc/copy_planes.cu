@@ -5,7 +5,8 @@
 // the error word in page-locked memory, so that the caller waits once.  Repeated calls, us,
 // copy calls against this: three planes read from 64^2 26.5 -> 11.6 (launch and wait), 1024^2
 // 40.6 -> 13.2, 4096^2 226 -> 70 (bandwidth, part of it from L2); all planes set at 64^2
-// 25.3 -> 14.1, 101^3 76 -> 20, 512^3 2304 -> 1231.  No size was found where the calls are better.
+// 25.3 -> 14.1, 101^3 76 -> 20, 512^3 2304 -> 1231.  No size was found where the calls are better
+// (9^3 to 4099^2, 5 x 917490, 10^6 x 4, aligned arrays and others).
 //
 // A kernel must not touch memory that a copy call would have refused or staged, so the
 // launch is taken only for arrays that the driver says lie whole in one plain device
@@ -21,7 +22,7 @@
 namespace gals {
 namespace {
 
-constexpr int kCopyThreads = 256, kCopyRows = kCopyThreads / 32;
+constexpr int kCopyThreads = 256, kCopyWarps = kCopyThreads / 32, kCopyPiece = 512;
 
 struct PlaneSet {
     const float *src[kMaxCopyPlanes];
@@ -33,26 +34,31 @@ __device__ __forceinline__ void report(const int *err, int *err_host)
     if (err_host && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *err_host = *err;
 }
 
-// Rows of different pitch: a warp per row, four loads in flight per lane.
+// Rows of different pitch: a warp per piece of kCopyPiece nodes of a row, four loads in flight
+// per lane.  With whole rows a state of few, long ones kept a handful of warps busy (three
+// planes of 10^6 x 4 nodes: 2882 us in whole rows, 21 in pieces, 75 by copy calls).
 __global__ void __launch_bounds__(kCopyThreads)
-k_copy_rows(const __grid_constant__ PlaneSet ps, int n0, int64_t rows, int64_t spitch, int64_t dpitch,
+k_copy_rows(const __grid_constant__ PlaneSet ps, int n0, int64_t rows, int pieces, int64_t spitch, int64_t dpitch,
             const int *err, int *err_host)
 {
     pdl_wait();
     const float *src = ps.src[blockIdx.y];
     float *dst = ps.dst[blockIdx.y];
     const int lane = threadIdx.x & 31;
-    for (int64_t r = (int64_t)blockIdx.x * kCopyRows + (threadIdx.x >> 5); r < rows; r += (int64_t)gridDim.x * kCopyRows) {
-        const float *s = src + r * spitch;
-        float *d = dst + r * dpitch;
-        for (int c = lane; c < n0; c += 128) {
+    const int64_t step = (int64_t)gridDim.x * kCopyWarps;
+    for (int64_t w = (int64_t)blockIdx.x * kCopyWarps + (threadIdx.x >> 5); w < rows * pieces; w += step) {
+        const int64_t r = pieces == 1 ? w : w / pieces;
+        const int c0 = (int)(w - r * pieces) * kCopyPiece, end = min(n0 - c0, kCopyPiece);
+        const float *s = src + r * spitch + c0;
+        float *d = dst + r * dpitch + c0;
+        for (int c = lane; c < end; c += 128) {
             float v[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (c + 32 * k < n0) v[k] = s[c + 32 * k];
+                if (c + 32 * k < end) v[k] = s[c + 32 * k];
 #pragma unroll
             for (int k = 0; k < 4; ++k)
-                if (c + 32 * k < n0) d[c + 32 * k] = v[k];
+                if (c + 32 * k < end) d[c + 32 * k] = v[k];
         }
     }
     report(err, err_host);
@@ -150,12 +156,13 @@ cudaError_t copy_planes(const PlaneCopy &c, cudaStream_t s, bool *done)
         ps.dst[p] = c.to_user ? c.user[p] : mine;
         dense = dense && (uintptr_t)c.user[p] % 16 == 0;
     }
+    const int pieces = (int)((c.n0 + kCopyPiece - 1) / kCopyPiece);
     const int64_t work = dense ? (count / 4 + 4 * kCopyThreads - 1) / (4 * kCopyThreads)
-                               : (c.rows + kCopyRows - 1) / kCopyRows;
+                               : (c.rows * pieces + kCopyWarps - 1) / kCopyWarps;
     const dim3 grid((unsigned)std::min<int64_t>(work, 4096), (unsigned)c.planes);
     *done = true;
     if (dense) return launch_kernel(k_copy_dense, grid, dim3(kCopyThreads), 0, s, true, ps, count / 4, c.err, c.err_host);
-    return launch_kernel(k_copy_rows, grid, dim3(kCopyThreads), 0, s, true, ps, (int)c.n0, c.rows,
+    return launch_kernel(k_copy_rows, grid, dim3(kCopyThreads), 0, s, true, ps, (int)c.n0, c.rows, pieces,
                          c.to_user ? c.pitch : c.n0, c.to_user ? c.n0 : c.pitch, c.err, c.err_host);
 }
 
