@@ -453,7 +453,7 @@ const char *gals_surrogate_last_error(const gals_surrogate *s);
  * not let cudaMalloc/cudaFree synchronise the device, or a service that accounts for
  * every byte it holds.  It computes what gals_diagnostics computes (same kernels), for
  * a state in caller memory, using a fixed scratch area inside the library (a
- * __device__ array of about 128 KB that each device holding the library keeps until
+ * __device__ array of about 144 KB that each device holding the library keeps until
  * the process exits) instead of allocating.
  *
  *   state       device pointer of plane 0 (plane order as above, all 4 / 8 planes with

@@ -77,6 +77,7 @@ struct gals_grid {
     int coef_cap = 0;
     DiagOut *diag_dev = nullptr;
     double *diag_partials = nullptr;
+    unsigned *diag_list = nullptr;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
     // gals_step_host: copy-in and copy-out streams, one event per band and direction
@@ -519,11 +520,13 @@ gals_status gals_create_grid(const gals_grid_desc *d, gals_grid **out)
         (e = cudaMalloc(&g->err_dev, sizeof(int))) != cudaSuccess ||
         (e = cudaMallocHost(&g->err_host, sizeof(int))) != cudaSuccess ||
         (e = cudaMalloc(&g->diag_dev, sizeof(DiagOut))) != cudaSuccess ||
-        (e = cudaMalloc(&g->diag_partials, sizeof(double) * diag_partials_needed())) != cudaSuccess) {
+        (e = cudaMalloc(&g->diag_partials, sizeof(double) * diag_partials_needed() + sizeof(unsigned) * kDiagList)) !=
+            cudaSuccess) {
         gals_status st = cuda_fail(nullptr, e, "cudaMalloc(aux)");
         gals_destroy_grid(g);
         return st;
     }
+    g->diag_list = reinterpret_cast<unsigned *>(g->diag_partials + diag_partials_needed());
 #ifdef GALS_CHECKED
     g->geom.chk = g->err_dev;  // the checked build's bounds errors land in the error word
 #endif
@@ -1137,7 +1140,7 @@ gals_status gals_diagnostics(gals_grid *g, const gals_diag_request *req, gals_di
         }
     }
     e = launch_diag(g->dim, g->geom, g->buf[g->cur], r ? r->buf[r->cur] : nullptr, req->q, g->diag_dev,
-                    g->diag_partials, g->stream, g->cross == GALS_CROSS_CELL,
+                    g->diag_partials, diag_partials_needed(), g->diag_list, g->stream, g->cross == GALS_CROSS_CELL,
                     r && r->cross == GALS_CROSS_CELL);
     if (e != cudaSuccess) return cuda_fail(g, e, "diagnostics launch");
     DiagOut h;

@@ -10,8 +10,9 @@
 // every device holding the library keeps until the process exits.  The caller passes the
 // state (and an optional reference) and receives the results; nothing is allocated.
 //
-// The scratch holds the result counters and one FP64 partial sum per block of the node
-// pass, one block per kNodesPerPartial nodes, so its capacity bounds the grid size.
+// The scratch holds the result counters, a list of the diagnostics' costly cells and one FP64
+// partial sum per block of the node pass, one block per kNodesPerPartial nodes, so its
+// capacity bounds the grid size.
 #include <cmath>
 #include <cstdint>
 #include <cstring>
@@ -30,11 +31,11 @@ constexpr int kMaxDevices = 64;
 
 struct Scratch {
     DiagOut counters;
-    double pad[3];
     double partials[kMaxPartials];
+    unsigned list[kDiagList];
 };
 
-// The scratch itself (about 128 KB per device).  In host code this name is only a
+// The scratch itself (about 144 KB per device).  In host code this name is only a
 // stand-in: its device address comes from cudaGetSymbolAddress, once per device (and
 // context).
 static __device__ __align__(256) unsigned char g_noalloc_scratch[sizeof(Scratch)];
@@ -155,9 +156,8 @@ gals_status gals_diagnostics_noalloc(int dim, const int *n, const double *lo, co
     // a block per partial: at least one per 1024 nodes up to the default number of blocks
     const int nparts = (int)std::max<int64_t>((nodes + kNodesPerPartial - 1) / kNodesPerPartial,
                                               std::min<int64_t>((nodes + 1023) / 1024, diag_partials_needed()));
-    // launch_diag_with clears the counters first: the scratch keeps the previous call's
-    // contents
-    e = launch_diag_with(dim, G, state, reference, q, &sc->counters, sc->partials, nparts, s);
+    // launch_diag clears the counters first: the scratch keeps the previous call's contents
+    e = launch_diag(dim, G, state, reference, q, &sc->counters, sc->partials, nparts, sc->list, s);
     if (e != cudaSuccess) return nfail(GALS_ERR_CUDA, cudaGetErrorString(e));
     DiagOut hcnt;
     if ((e = cudaMemcpyAsync(&hcnt, &sc->counters, sizeof(hcnt), cudaMemcpyDeviceToHost, s)) != cudaSuccess ||

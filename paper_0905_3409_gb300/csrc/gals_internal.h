@@ -141,15 +141,16 @@ struct DiagOut {
     unsigned long long n_neg, n_sym, nonfinite;
     unsigned int emax_phi_bits, emax_psi_bits;  // non-negative floats as ordered integers
     double l2_phi_sum;
+    unsigned int dense, pad;                 // warps with many undecided cells
+    unsigned long long pre_neg, pre_sym;     // what the pass that finds them counts
 };
-// Scratch: `partials` holds at least diag_partials_needed() doubles; `counters` a DiagOut.
-int diag_partials_needed();
+// The diagnostics' launches with `nparts` blocks (one FP64 partial each; diag_partials_needed()
+// unless the caller has a reason).  Scratch: nparts doubles, a DiagOut, kDiagList words.
 // cell_a / cell_b: the interpolant of a / b takes its mixed derivatives by approach B.
-cudaError_t launch_diag(int dim, const Geom &g, const float *a, const float *b, int q,
-                        DiagOut *counters, double *partials, cudaStream_t s, bool cell_a = false,
+constexpr unsigned kDiagList = 4096;
+int diag_partials_needed();
+cudaError_t launch_diag(int dim, const Geom &g, const float *a, const float *b, int q, DiagOut *counters,
+                        double *partials, int nparts, unsigned *list, cudaStream_t s, bool cell_a = false,
                         bool cell_b = false);
-// Same kernels with `nparts` node blocks (one FP64 partial each) instead of the default.
-cudaError_t launch_diag_with(int dim, const Geom &g, const float *a, const float *b, int q,
-                             DiagOut *counters, double *partials, int nparts, cudaStream_t s);
 
 }  // namespace gals
