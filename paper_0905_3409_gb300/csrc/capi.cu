@@ -72,7 +72,7 @@ struct gals_grid {
     char *pt_buf = nullptr;       // gals_eval_points: device staging of host points / results
     size_t pt_cap = 0;
     int *err_dev = nullptr;       // device error word written by kernels (bounded waits)
-    int *err_host = nullptr;      // its page-locked copy, filled on the stream before a wait
+    HostWord err_word;      // its page-locked copy (host_word.h), filled on the stream before a wait
     StageCoef *coef = nullptr;    // per-step stage coefficients of the current call
     int coef_cap = 0;
     DiagOut *diag_dev = nullptr;
@@ -518,7 +518,7 @@ gals_status gals_create_grid(const gals_grid_desc *d, gals_grid **out)
     }
     if ((e = cudaMalloc(&g->t_dev, sizeof(double))) != cudaSuccess ||
         (e = cudaMalloc(&g->err_dev, sizeof(int))) != cudaSuccess ||
-        (e = cudaMallocHost(&g->err_host, sizeof(int))) != cudaSuccess ||
+        (e = acquire_host_word(&g->err_word)) != cudaSuccess ||
         (e = cudaMalloc(&g->diag_dev, sizeof(DiagOut))) != cudaSuccess ||
         (e = cudaMalloc(&g->diag_partials, sizeof(double) * diag_partials_needed() + sizeof(unsigned) * kDiagList)) !=
             cudaSuccess) {
@@ -583,7 +583,7 @@ gals_status gals_destroy_grid(gals_grid *g)
     for (int b = 0; b < 2; ++b) cudaFree(g->buf[b]);
     cudaFree(g->t_dev);
     cudaFree(g->err_dev);
-    cudaFreeHost(g->err_host);
+    release_host_word(g->err_word);
     cudaFree(g->trace_buf);
     cudaFree(g->pt_buf);
     cudaFree(g->coef);
@@ -851,7 +851,7 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
 static gals_status wait_and_check(gals_grid *g, const char *what, bool copied = false)
 {
     int code = 0;
-    const cudaError_t e = fetch_error_word(g->err_dev, g->err_host, g->stream, copied, &code);
+    const cudaError_t e = fetch_error_word(g->err_dev, g->err_word.at, g->stream, copied, &code);
     if (e != cudaSuccess) return cuda_fail(g, e, what);
     if (code == 0) return GALS_OK;
     if ((code & 0xff) == kErrBounds)
@@ -903,7 +903,7 @@ gals_status gals_read_state(gals_grid *g, float *const *fields, int nfields, int
     bool copied = false;
     if (memspace == GALS_MEM_DEVICE) {
         const PlaneCopy c{g->buf[g->cur], G.plane, G.pitch, g->n[0], (int64_t)rows, fields, nfields, true,
-                          g->err_dev, g->err_host};
+                          g->err_dev, g->err_word.at};
         if ((e = copy_planes(c, g->stream, &copied)) != cudaSuccess) return cuda_fail(g, e, "read_state copy");
     }
     for (int p = 0; p < nfields && !copied; ++p) {

@@ -56,7 +56,7 @@ struct gals_batch {
     StageCoef *coef = nullptr;
     int64_t coef_cap = 0;
     int *err_dev = nullptr;
-    int *err_host = nullptr;               // page-locked copy of the error word
+    HostWord err_word;               // page-locked copy of the error word
     int cur = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
@@ -247,7 +247,7 @@ cudaError_t issue(gals_batch *b, int kind, int nsteps)
 gals_status wait_and_check(gals_batch *b, const char *what, bool copied = false)
 {
     int code = 0;
-    const cudaError_t e = fetch_error_word(b->err_dev, b->err_host, b->stream, copied, &code);
+    const cudaError_t e = fetch_error_word(b->err_dev, b->err_word.at, b->stream, copied, &code);
     if (e != cudaSuccess) return bcuda(b, e, what);
     if (code == 0) return GALS_OK;
     if ((code & 0xff) == kErrBounds)
@@ -336,7 +336,7 @@ gals_status gals_create_batch(const gals_grid_desc *descs, int count, gals_batch
         (e = cudaMalloc(&b->vps_dev, sizeof(VelParams) * count)) != cudaSuccess ||
         (e = cudaMalloc(&b->t_dev, sizeof(double) * count)) != cudaSuccess ||
         (e = cudaMalloc(&b->err_dev, sizeof(int))) != cudaSuccess ||
-        (e = cudaMallocHost(&b->err_host, sizeof(int))) != cudaSuccess)
+        (e = acquire_host_word(&b->err_word)) != cudaSuccess)
         return bail(e, "cudaMalloc(descriptors)");
     if ((e = cudaMemsetAsync(b->err_dev, 0, sizeof(int), b->stream)) != cudaSuccess) return bail(e, "cudaMemset");
 #ifdef GALS_CHECKED
@@ -436,7 +436,7 @@ gals_status gals_destroy_batch(gals_batch *b)
     cudaFree(b->t_dev);
     cudaFree(b->coef);
     cudaFree(b->err_dev);
-    cudaFreeHost(b->err_host);
+    release_host_word(b->err_word);
     if (b->own_stream && b->stream) cudaStreamDestroy(b->stream);
     delete b;
     return GALS_OK;
@@ -563,7 +563,7 @@ gals_status gals_batch_read_state(gals_batch *b, int index, float *const *fields
     const cudaMemcpyKind kind = memspace == GALS_MEM_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     bool copied = false;
     if (memspace == GALS_MEM_DEVICE) {
-        const PlaneCopy c{src, G.plane, G.pitch, G.n0, G.n1, fields, nfields, true, b->err_dev, b->err_host};
+        const PlaneCopy c{src, G.plane, G.pitch, G.n0, G.n1, fields, nfields, true, b->err_dev, b->err_word.at};
         if ((e = copy_planes(c, b->stream, &copied)) != cudaSuccess) return bcuda(b, e, "read_state copy");
     }
     for (int p = 0; p < nfields && !copied; ++p)

@@ -7,6 +7,7 @@
 
 #include "../../include/gals.h"
 #include "gals_internal.h"
+#include "host_word.h"
 #include "mlp_internal.h"
 
 #include <nvtx3/nvToolsExt.h>

@@ -47,30 +47,6 @@ struct ScratchSlot {
 };
 ScratchSlot g_slot[kMaxDevices];
 
-// Unique id of the driver's current context (cuCtxGetCurrent, cuCtxGetId; reached through
-// the runtime's driver entry points so that the library links against the runtime only);
-// 0 when no context is current or the driver does not offer the calls.  Ids are never
-// reused within a process, unlike context handles.
-unsigned long long current_context_id()
-{
-    typedef int (*CtxGetCurrent)(void **);
-    typedef int (*CtxGetId)(void *, unsigned long long *);
-    auto entry = [](const char *name) -> void * {
-        void *p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion(name, &p, 12000, cudaEnableDefault, &q) != cudaSuccess ||
-            q != cudaDriverEntryPointSuccess)
-            return nullptr;
-        return p;
-    };
-    static CtxGetCurrent get_current = reinterpret_cast<CtxGetCurrent>(entry("cuCtxGetCurrent"));
-    static CtxGetId get_id = reinterpret_cast<CtxGetId>(entry("cuCtxGetId"));
-    void *ctx = nullptr;
-    unsigned long long id = 0;
-    if (!get_current || !get_id || get_current(&ctx) != 0 || !ctx || get_id(ctx, &id) != 0) return 0;
-    return id;
-}
-
 // Device address of the scratch on the current device.  The lookup
 // (cudaGetSymbolAddress) is the set-up: it runs on the first call on a device, and again
 // only if that device's context has changed since (after cudaDeviceReset, or when the
