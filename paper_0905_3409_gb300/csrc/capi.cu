@@ -156,17 +156,29 @@ gals_status make_velparams(gals_grid *g, const gals_velocity *v, VelParams &vp)
 // Whether the steps of a FULL 3D run rebuild the mixed derivatives (step_launch): while few
 // feet leave the staged tile, one cell around it.  The deformation field's bound is reached
 // by one component at a few nodes (half of it stands for the field), a rotation's by an
-// edge of the box.  Measured, us per step, rebuilt against reconstructed: 256^3 deformation
+// edge of the box; of a constant field every foot lies equally far, one whole cell up already in
+// the cell beyond, and along x the staged tile has three cells to spare.  Measured, us per step, rebuilt against reconstructed: 256^3 deformation
 // at CFL 1 / 2 / 4 344 against 351, 345 against 352, 386 against 379; rotation at CFL 1 / 2
-// 306 against 311, 450 against 398; 101^3 deformation at CFL 2 33.2 against 37.4.
+// 306 against 311, 450 against 398; 101^3 deformation at CFL 2 33.2 against 37.4; 256^3 constant
+// at CFL 0.5 281 against 284, at CFL 1 456 against 371.
 // The Heun form evaluates a velocity more after the interpolant and has no registers to
 // spare there: above a few million nodes, where the saved launch does not count, it keeps the
 // pass (200 x 190 x 180 deformation 167 us against 161, rotation 142 against 134; 101^3 33.7
-// against 36.1).
-bool rebuild3d(int kind, int trace, int64_t nodes, double reach)
+// against 36.1), as does a rotation with the Euler trace, whose step is short beside the
+// rebuilding (200 x 190 x 180 140 against 132; 101^3 31 against 34).
+bool rebuild3d(const gals_grid *g, const gals_velocity *v, double dt, double vmax)
 {
-    return (kind == GALS_VEL_DEFORM3D ? 0.5 * reach : reach) <= 1.05 &&
-           (trace != GALS_TRACE_HEUN_PSI || nodes <= 2000000);
+    const double reach = dt * vmax / std::min({g->h[0], g->h[1], g->h[2]});
+    if (v->kind == GALS_VEL_CONST) {
+        if (dt * std::max({std::fabs(v->c[0]) / (3.0 * g->h[0]), std::fabs(v->c[1]) / g->h[1],
+                           std::fabs(v->c[2]) / g->h[2]}) > 0.999)
+            return false;
+    } else if ((v->kind == GALS_VEL_DEFORM3D ? 0.5 * reach : reach) > 1.05) {
+        return false;
+    }
+    const bool heavy = v->trace == GALS_TRACE_HEUN_PSI ||
+                       (v->trace == GALS_TRACE_EULER && v->kind == GALS_VEL_ROTATION);
+    return !heavy || (int64_t)g->n[0] * g->n[1] * g->n[2] <= 2000000;
 }
 
 // Kernel launch descriptor of step s of a run of nsteps, from buffer cur to buffer cur ^ 1.
@@ -739,8 +751,7 @@ gals_status gals_step(gals_grid *g, const gals_velocity *v, double dt, int nstep
     }
     const double vmax = speed_bound(v, g->dim, g->lo, g->hi);
     const double reach[2] = {dt * vmax / g->h[0], dt * vmax / g->h[1]};
-    const bool rebuild = g->dim == 2 || rebuild3d(v->kind, v->trace, (int64_t)g->n[0] * g->n[1] * g->n[2],
-                                                      std::max({reach[0], reach[1], dt * vmax / g->h[2]}));
+    const bool rebuild = g->dim == 2 || rebuild3d(g, v, dt, vmax);
     const bool run = use_run(g, v->trace, std::min(nsteps, kGraphSteps), reach);
     if (run && !g->run_ctl) {
         if ((e = cudaStreamSynchronize(g->stream)) != cudaSuccess) return cuda_fail(g, e, "sync");
