@@ -78,8 +78,15 @@ __device__ __forceinline__ void stage_yz(float *tile, const Geom &g, int y0)
 // passes: 256^3 deformation 344 against 447 / 351, rotation 306 against 406 / 311, 101^3
 // deformation 33.2 against 39.8 / 37.4.  Tiles of 2, 6 or 8 levels (363, 354, 356) and a halo
 // of two cells (397) were slower, as was a branch for the one-sided ends per difference (373).
-template <int TR, int VK, int CR>
-__global__ void __launch_bounds__(TX *TY, CR == CROSS_CELL ? 1 : 4)
+// WIDE (CROSS_RECON on grids that put at most two blocks on an SM, step3d_wide): twice the
+// registers, and feet outside the tile both at once, all their values from global memory (a
+// choice per value cost 30 us of 150).  There a step is the latency of one block; us per step with
+// one foot after the other / the windows of both before that / now: 48^3 constant at CFL 2
+// 12.5 / 9.2 / 7.5, rotation at CFL 6 15.9 / 12.9 / 9.9, deformation at CFL 0.5 7.7 / 7.6 / 6.3;
+// 33 x 30 x 28 deformation 6.2 / 5.8 / 5.6.  At 390 blocks (64 x 60 x 50) it loses: rotation at
+// CFL 2 18.0 against 14.9.
+template <int TR, int VK, int CR, bool WIDE>
+__global__ void __launch_bounds__(TX *TY, CR == CROSS_CELL ? 1 : (WIDE ? 2 : 4))
 k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParams vp,
          const StageCoef *__restrict__ coef, float dt, const __grid_constant__ CUtensorMap tmap,
          int *__restrict__ err, int zlo)
@@ -115,6 +122,16 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
         const int kz1 = two ? kz + 1 : kz;
         const F2 Z = make_float2(g.lo2 + (float)kz * g.h2, g.lo2 + (float)kz1 * g.h2);
         F2 d[3], J[9];
+        auto trace = [&]() {
+            if (kz + 2 >= zend) pdl_release();
+            trace3d_pair<TR, VK>(stage1_pair<VK>(vp, sc, pre, X, Y, Z), vp, sc, X, Y, Z, dt, d, J);
+            if (JS)
+#pragma unroll
+                for (int e = 0; e < 9; ++e) Jsh[e][tid] = J[e];
+        };
+        // CROSS_RECON: the first trace while the tile is on its way (33 x 30 x 28 deformation 6.2 ->
+        // 5.7 us per step, large grids the same)
+        if (CR == CROSS_RECON) trace();
         if (kz == z0) {
             if (!mbar_wait_block(&bar, 0)) {
                 if (tid == 0) {
@@ -128,12 +145,7 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
                 __syncthreads();
             }
         }
-        if (kz + 2 >= zend) pdl_release();
-        trace3d_pair<TR, VK>(stage1_pair<VK>(vp, sc, pre, X, Y, Z), vp, sc, X, Y, Z, dt, d, J);
-
-        if (JS)
-#pragma unroll
-            for (int e = 0; e < 9; ++e) Jsh[e][tid] = J[e];
+        if (CR != CROSS_RECON) trace();
 
         int k0, l0, m0, k1, l1, m1;
         float xi0, eta0, zeta0, xi1, eta1, zeta1;
@@ -232,10 +244,13 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
                 hermite3d_pair(bx, by, bz, [&](int G, int B, int C, F2 lo[4], F2 hi[4]) { line(G, B, C, lo, hi, true); }, H, gr);
             else
                 hermite3d_pair(bx, by, bz, [&](int G, int B, int C, F2 lo[4], F2 hi[4]) { line(G, B, C, lo, hi, false); }, H, gr);
-        } else if (CR == CROSS_RECON) {
-            // a foot outside the tile: both from global memory, one at a time (both lanes the same
-            // foot), so that this path's windows do not set the kernel's registers
-#pragma unroll 1
+        } else if (CR == CROSS_RECON && !WIDE) {
+            // a foot outside the tile: both from global memory, a foot's two lanes the same, so that
+            // this path's windows do not set the kernel's registers; one at a time where two would
+            // all the same (256^3, us per step: constant at CFL 2 574 one at a time, 503 both; RK3
+            // deformation 348 against 354)
+            constexpr int kFeet = VK == VK_DEFORM3D && TR == TR_RK3 ? 1 : 2;
+#pragma unroll kFeet
             for (int e = 0; e < 2; ++e) {
                 const int k = e ? k1 : k0, l = e ? l1 : l0, m = e ? m1 : m0;
                 auto dup = [&](const F2 &v) { return bc(e ? v.y : v.x); };
@@ -274,8 +289,9 @@ k_step3d(const float *__restrict__ in, float *__restrict__ out, Geom g, VelParam
                 }
             }, H, gr);
         } else {
-            auto ld0 = [&](int a, int zz, int yy, int xx) { return in0 ? lds(a, zz, yy, xx) : ldg(a, zz, yy, xx); };
-            auto ld1 = [&](int a, int zz, int yy, int xx) { return in1 ? lds(a, zz, yy, xx) : ldg(a, zz, yy, xx); };
+            // (WIDE: both feet from global memory, without the choice per value)
+            auto ld0 = [&](int a, int zz, int yy, int xx) { return !WIDE && in0 ? lds(a, zz, yy, xx) : ldg(a, zz, yy, xx); };
+            auto ld1 = [&](int a, int zz, int yy, int xx) { return !WIDE && in1 ? lds(a, zz, yy, xx) : ldg(a, zz, yy, xx); };
             hermite3d_lines(bx, by, bz, [&](int B, int C, F2 lo[8], F2 hi[8]) {
                 float a0[8], b0[8], a1[8], b1[8];
                 cell_line<CR>(ld0, g, k0, l0, m0, B, C, a0, b0);
@@ -425,17 +441,24 @@ k_recon3d_tma(float *__restrict__ buf, Geom g, const __grid_constant__ CUtensorM
     }
 }
 
-template <int TR, int VK, int CR>
+// Whether a step has at most two blocks for each of the chip's 152 SMs (whole grid, so that every
+// band decides alike).
+bool step3d_wide(const Geom &g)
+{
+    return (int64_t)((g.n0 + TX - 1) / TX) * ((g.n1 + TY - 1) / TY) * ((g.n2 + TZ - 1) / TZ) <= 2 * 152;
+}
+
+template <int TR, int VK, int CR, bool WIDE = false>
 cudaError_t launch_t(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
     using T = Tile3<CR>;
     static PerDevice ready;
-    cudaError_t e = ready.once([] { return allow_dynamic_smem(k_step3d<TR, VK, CR>, T::SMEM); });
+    cudaError_t e = ready.once([] { return allow_dynamic_smem(k_step3d<TR, VK, CR, WIDE>, T::SMEM); });
     if (e != cudaSuccess) return e;
     dim3 block(TX, TY);
     dim3 grid((a.geom.n0 + TX - 1) / TX, (a.geom.n1 + TY - 1) / TY, (z1 - z0 + TZ - 1) / TZ);
     const CUtensorMap &map = *a.tmap[0][CR == CROSS_PLANE];
-    return launch_kernel(k_step3d<TR, VK, CR>, grid, block, T::SMEM, s, a.dependent, a.in, a.out, a.geom, a.vp, a.coef,
+    return launch_kernel(k_step3d<TR, VK, CR, WIDE>, grid, block, T::SMEM, s, a.dependent, a.in, a.out, a.geom, a.vp, a.coef,
                          (float)a.dt, map, a.err, z0);
 }
 
@@ -443,8 +466,9 @@ template <int TR, int VK>
 cudaError_t launch_cr(const StepLaunch &a, cudaStream_t s, int z0, int z1)
 {
     if (a.cross_in == CROSS_CELL) return launch_t<TR, VK, CROSS_CELL>(a, s, z0, z1);
-    return a.cross_in == CROSS_PLANE ? launch_t<TR, VK, CROSS_PLANE>(a, s, z0, z1)
-                                     : launch_t<TR, VK, CROSS_RECON>(a, s, z0, z1);
+    if (a.cross_in == CROSS_PLANE) return launch_t<TR, VK, CROSS_PLANE>(a, s, z0, z1);
+    return step3d_wide(a.geom) ? launch_t<TR, VK, CROSS_RECON, true>(a, s, z0, z1)
+                               : launch_t<TR, VK, CROSS_RECON>(a, s, z0, z1);
 }
 
 template <int VK>
