@@ -10,7 +10,7 @@
 // the SM count) the blocks are persistent and re-use their shared memory and barrier
 // (one mbarrier phase per tile).
 #include "batch_internal.h"
-#include "step2d_walk.cuh"
+#include "step2d_tile.cuh"
 
 namespace gals {
 
@@ -18,16 +18,10 @@ namespace {
 
 using namespace t2;
 
-// Whether the steps that write no phi_xy walk their tiles (as on one grid: the Fourier field's
-// tables leave no registers for the carried rows).
-template <int VK, int WC> constexpr bool walked() { return !WC && VK != VK_FOURIER2D; }
-
-template <int TY, int VK, int WC> struct BatchSmemOf { using T = Smem<TY, WC>; };
-template <int TY> struct BatchSmemOf<TY, VK_VORTEX2D, 0> { using T = WalkSmem<TY>; };
-template <int TY> struct BatchSmemOf<TY, VK_ROTATION, 0> { using T = WalkSmem<TY>; };
-
 // Blocks per SM: the steps between the first and the last of a run (no phi_xy plane, no
-// exchange of psi_y) fit five.
+// exchange of psi_y) fit five.  They don't walk their tiles as on one grid: on problems of the
+// batch's sizes the walk is slower (64 problems of 256^2, COMPACT vortex 54.1 us per step
+// walked, 51.1 not; 24 of 100 to 260 nodes a side 21.6 and 19.7; 6 of 1024^2 57.8 and 57.7).
 template <int TY, int VK, int CR, int WC>
 __global__ void __launch_bounds__(TX, WC ? 4 : 5)
 k_batch2d(const float *__restrict__ in_base, float *__restrict__ out_base,
@@ -36,7 +30,7 @@ k_batch2d(const float *__restrict__ in_base, float *__restrict__ out_base,
           const BatchItem *__restrict__ items, int nitems, int *__restrict__ err)
 {
     extern __shared__ __align__(128) float tile[];
-    __shared__ __align__(16) typename BatchSmemOf<TY, VK, WC>::T sm;
+    __shared__ __align__(16) Smem<TY, WC> sm;
     if (threadIdx.x == 0) mbar_init(&sm.bar, 1);
     __syncthreads();
     uint32_t parity = 0;
@@ -44,15 +38,9 @@ k_batch2d(const float *__restrict__ in_base, float *__restrict__ out_base,
         const BatchItem w = items[it];
         const BatchProb &P = probs[w.prob];
         const Geom g = P.g;
-        bool ok;
-        if constexpr (walked<VK, WC>())
-            ok = tile_walk2d<TY, TR_RK3, VK, CR, HY, TW>(in_base + P.off, out_base + P.off, g, vps[w.prob],
-                                                         coef + w.prob, P.dt, maps + w.prob, err, w.x0, w.y0, g.n1,
-                                                         tile, sm, parity);
-        else
-            ok = tile_step2d<TY, TR_RK3, VK, CR, WC>(in_base + P.off, out_base + P.off, g, vps[w.prob],
-                                                     coef + w.prob, P.dt, maps + w.prob, err, w.x0, w.y0, tile, sm,
-                                                     parity);
+        const bool ok = tile_step2d<TY, TR_RK3, VK, CR, WC>(
+            in_base + P.off, out_base + P.off, g, vps[w.prob], coef + w.prob, P.dt,
+            maps + w.prob, err, w.x0, w.y0, tile, sm, parity);
         if (!ok) return;  // block-uniform
         parity ^= 1u;
         __syncthreads();  // tile and psi_y buffers are free before the next copy
