@@ -319,13 +319,14 @@ def pinned_near_gpu(local, arrays):
     return pins, info
 
 
-# the sources that define each benchmarked kernel: a recorded DRAM traffic figure is
-# reported only while these files are unchanged
+# the sources that define each benchmarked step, the kernels and the rules that choose among them
+# (capi.cu) with every file these include: a recorded DRAM traffic figure is reported only while
+# they are unchanged
+STEP_COMMON = ["capi.cu", "gals_device.cuh", "gals_internal.h", "gals_pair.cuh", "per_device.h", "tma.cuh"]
 KERNEL_SOURCES = {
     2: ["step2d.cu", "step2d_fourier.cu", "step2d_kernels.cuh", "step2d_kinds.h", "step2d_linear.cu",
-        "step2d_small.cu", "step2d_tile.cuh", "step2d_vortex.cu", "step2d_walk.cuh", "step2d_waves.cu",
-        "gals_pair.cuh", "gals_device.cuh", "tma.cuh", "capi.cu"],
-    3: ["step3d.cu", "step3d_common.cuh", "gals_pair.cuh", "gals_device.cuh", "tma.cuh"],
+        "step2d_small.cu", "step2d_tile.cuh", "step2d_vortex.cu", "step2d_walk.cuh", "step2d_waves.cu"] + STEP_COMMON,
+    3: ["step3d.cu", "step3d_common.cuh"] + STEP_COMMON,
 }
 
 
