@@ -77,8 +77,10 @@ cudaError_t launch_step2d_run(const RunLaunch &a, cudaStream_t s);
 // (small2d_fits): at most kSmallNodes nodes in rows of at most kSmallColumns, and the
 // blocks' shared memory; a run of at least kSmallSteps steps.  At every size up to the limit
 // it is the faster way (128 x 96: 1.8 us per step against 7.2 for the banded launches;
-// 512 x 24: 2.4 against 6.7); larger grids keep the launches per step and band that
-// gals_last_step_launches is specified to count, and a run of fewer than 8 steps gains
+// 512 x 24: 2.4 against 6.7).  It does not stop being faster there: 128 x 97 takes 7.2, and the
+// shared memory would hold four times the nodes.  The limit is the interface's: larger grids keep
+// the launches per step and band that gals_last_step_launches is specified to count.  A run of
+// fewer than 8 steps gains
 // little, its coefficient and clock kernels being most of it (5.3 us per step at 8 steps
 // against 9.9 at 7 of a first launch per step).
 constexpr int kSmallNodes = 12288, kSmallColumns = 512, kSmallSteps = 8;

@@ -333,7 +333,8 @@ __device__ __forceinline__ bool tile_fails(const InferParams &ip, const Geom &g,
 // A costly field keeps the check in the group, a sample per warp with its modes over the
 // lanes: one warp alone falls behind the network.  2048^2, us per step in the group / aside:
 // 256 waves, 4 nodes 926 / 811, 16 nodes 1397 / 2259, every tile failing 3443 / 3996; 1024
-// waves, 4 nodes 1382 / 2262.
+// waves, 4 nodes 1382 / 2262.  The rule looks at the kind of field alone: with few waves and
+// nodes aside gains up to 1.14 times, with more of either it costs up to 1.64.
 template <int VK> constexpr bool aside() { return VK != VK_WAVES2D; }
 
 template <int VK>

@@ -187,8 +187,9 @@ k_step2d_run(float *__restrict__ buf0, float *__restrict__ buf1, Geom g, VelPara
 // Whether the grid has too few tall tiles to occupy the chip (whole grid, so that every band
 // of a step decides alike): a short tile then does in one row pair per thread what a tall
 // one does in seven, on seven times the blocks, its trace hidden behind the tile's copy.
-// The line is at about one wave of tall tiles (5 blocks on each of 152 SMs).  Measured, us
-// per step, short against tall tiles: vortex 200 x 172 2.8 against 6.8, 1021 x 777 (448 tall
+// The line, 850 tall tiles, lies between the largest grid measured faster with short ones (747)
+// and the smallest measured faster with tall ones (1023); a full wave of them, five blocks on
+// each of 152 SMs, is 760.  Us per step, short against tall tiles: vortex 200 x 172 2.8 against 6.8, 1021 x 777 (448 tall
 // tiles) 6.8 against 8.9, 1150^2 (747) 10.9 against 12.0, 1300^2 (1023) 14.5 against 13.7,
 // 2048^2 34.1 against 27.5; rotation 1150^2 9.2 against 9.5, 1300^2 12.1 against 11.0.
 bool short_tiles(const Geom &g)

@@ -2,6 +2,8 @@
 cached graphs or the small grids' cluster run and moves the host's clock, is refused, on a
 small grid as on a larger one, and leaves the grid as it was; the same call after the
 capture steps as on a grid that was never captured."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -34,17 +36,18 @@ def test_several_steps_are_refused_while_captured(G, n, steps):
         g.step(vel, dt, steps)          # tables and attributes are there before the capture
         g.synchronize()
     t, launches = a.time, a.last_step_launches()
-    graph = torch.cuda.CUDAGraph()
-    with torch.cuda.stream(stream):
-        graph.capture_begin()
-        try:
-            with pytest.raises(G.GalsError) as e:
-                a.step(vel, dt, steps)
-        finally:
-            try:
-                graph.capture_end()
-            except RuntimeError:
-                pass                    # the refused call may have ended the capture
+    # by the runtime itself: a capture that the refused call ends early would leave torch's
+    # allocator waiting for the end of it
+    rt, graph, s = ctypes.CDLL("libcudart.so.13"), ctypes.c_void_p(), ctypes.c_void_p(stream.cuda_stream)
+    assert rt.cudaStreamBeginCapture(s, ctypes.c_int(1)) == 0  # thread-local mode
+    try:
+        with pytest.raises(G.GalsError) as e:
+            a.step(vel, dt, steps)
+    finally:
+        rt.cudaStreamEndCapture(s, ctypes.byref(graph))
+        if graph:
+            rt.cudaGraphDestroy(graph)
+        rt.cudaGetLastError()
     assert e.value.status == G.ERR_CUDA
     assert a.time == t
     assert np.array_equal(a.read_state(), b.read_state())
