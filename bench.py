@@ -341,9 +341,10 @@ def kernel_source_hash(dim=None):
     return h.hexdigest()[:16]
 
 
-def recorded_traffic(workload, layout):
-    """DRAM bytes per launch of the step kernel from the committed ncu summary, if it was
-    taken on the current kernel sources; else None."""
+def recorded_traffic(workload, layout, steps):
+    """DRAM bytes per step from the committed ncu summary, if it was taken on the current
+    kernel sources (else None): the mean over a call of `steps` steps, an inner step's bytes
+    and what the first and the last step of each run of at most 256 steps move beyond them."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
@@ -352,7 +353,7 @@ def recorded_traffic(workload, layout):
     e = d.get(f"{workload}/{layout}")
     if not e or e.get("kernel_sources") != kernel_source_hash(WORKLOADS[workload]["dim"]):
         return None
-    return e.get("dram_bytes_per_launch")
+    return round(e["dram_bytes_inner_step"] + e["dram_bytes_run_ends"] * math.ceil(steps / 256) / steps)
 
 
 # ---------------------------------------------------------------------- CPU oracle leg
@@ -559,7 +560,7 @@ def run_batch(args, wl):
                        "timing": "median of repeated K-step windows", "windows": window_summary(wins),
                        "parallelism": f"{world} independent replica(s), one per GPU"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                         "frac": achieved / peak, "traffic": recorded_traffic(args.workload, args.layout),
+                         "frac": achieved / peak, "traffic": recorded_traffic(args.workload, args.layout, args.steps),
                          "peak_source": peak_kind, "kernel": "k_batch2d (1 launch per step)"},
             "e2e": {"value": nodes * e2e_steps / el, "unit": UNIT, "h2d_bytes_per_step": io_bytes,
                     "d2h_bytes_per_step": io_bytes},
@@ -716,7 +717,7 @@ def run_ours(args, wl):
                        "parallelism": f"{world} independent replica(s), one per GPU"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak,
-                         "traffic": recorded_traffic(args.workload, args.layout) if default_path else None,
+                         "traffic": recorded_traffic(args.workload, args.layout, args.steps) if default_path else None,
                          "peak_source": peak_kind,
                          "kernel": ("k_step2d_run (persistent: the K steps in one launch)" if persistent
                                     else f"gals step ({call_launches} kernel launches per "
@@ -801,7 +802,7 @@ def secondary_3d(args, R, local, stream):
             "windows": window_summary(wins),
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "peak_source": peak_kind,
-                         "traffic": recorded_traffic("deform512", "full"),
+                         "traffic": recorded_traffic("deform512", "full", K),
                          "kernel": "k_step3d (k_recon3d_tma after a call's last step)"},
             "gpu_launches_per_window": launches, "clocks": clocks}
 
