@@ -251,8 +251,10 @@ k_diag(Geom g, int lx_, const float *__restrict__ a, const float *__restrict__ b
         const Place P = place_of<DIM>(g, lx, it, threadIdx.x);
         const int64_t o = P.at;
         const bool look = q > 0 && noted <= limit;
-        // at items 2, 4, 8, 16, 24, ... and for the next one (at every item the read cost 15 of 48 us)
-        if (q > 0 && ((++turn & 7) == 0 || turn == 2 || turn == 4)) noted = *(volatile unsigned *)&out->dense;
+        // at items 2, 4, 8, 16, 24, ... and for the next one (at every item the read cost 15 of 48 us);
+        // one lane's reading for the whole warp, whose lanes have to look alike (the votes below)
+        if (q > 0 && ((++turn & 7) == 0 || turn == 2 || turn == 4))
+            noted = __shfl_sync(0xffffffffu, *(volatile unsigned *)&out->dense, 0);
         if (P.node) {
             bool bad = false;
 #pragma unroll
